@@ -17,7 +17,9 @@
 // list; pass B (k_frame_bin) appends uniform tiles to their material's list and
 // packs mixed-tile pixels into their material's 128-slot tiles (warp-aggregated
 // atomics: one atomic per material present in a warp).  Then the decode kernel
-// runs over those chunks.  All four launches are captured in one CUDA graph.
+// runs over those chunks.  Between the passes k_frame_texels decodes the visible
+// materials' latent texels once (see the rule at frame_texels_rule).  All the
+// launches are captured in one CUDA graph.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -177,6 +179,61 @@ __global__ void k_frame_bin(FrameDev F) {
   }
 }
 
+// ---- decoded latent texels of a frame
+//
+// A run of consecutive BC1 blocks of one material's level (its mips back to back).
+struct TexelRun {
+  int mat, level;
+  int first, count;  // blocks, count <= kTexelRun
+};
+constexpr int kTexelRun = 256;
+
+// One thread per block of a run: the block's four palette colours, then its 16
+// texels as RGBA8 words, four 16-byte row stores (neighbouring threads write
+// neighbouring 16 bytes of a row).  Materials without a pixel in this frame (the
+// counts of pass A) are left out.  Bound by its writes, 4 bytes per latent texel:
+// the 7.0 M texels of 64 materials up to 2048^2 take 9.9 us.
+__global__ void __launch_bounds__(kTexelRun) k_frame_texels(const TexelRun* __restrict__ runs, const MatDev* __restrict__ mats,
+                                                            FrameDev F) {
+  const TexelRun R = runs[blockIdx.x];
+  if (F.ucount[R.mat] + F.pcount[R.mat] == 0) return;
+  if ((int)threadIdx.x >= R.count) return;
+  const MatDev& M = mats[R.mat];
+  const int g = R.first + (int)threadIdx.x;  // block of the level, over its mips
+  int m = 0;
+  while (m + 1 < M.mips[R.level] && g >= M.mip_off[R.level][m + 1]) ++m;
+  const LevelView V = mip_view(M, R.level, m);
+  const int b = g - M.mip_off[R.level][m];
+  const int by = b / V.wb, bx = b - by * V.wb;
+  const uint64_t blk = __ldg(V.blocks + block_index(V, bx, by));
+  const uint32_t c0 = (uint32_t)(blk & 0xFFFFu), c1 = (uint32_t)((blk >> 16) & 0xFFFFu), bits = (uint32_t)(blk >> 32);
+  const bool four = c0 > c1;
+  int e0[3], e1[3];
+  expand565(c0, e0[0], e0[1], e0[2]);
+  expand565(c1, e1[0], e1[1], e1[2]);
+  uint32_t p[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    p[0] |= (uint32_t)e0[c] << (8 * c);
+    p[1] |= (uint32_t)e1[c] << (8 * c);
+    p[2] |= (uint32_t)palette_channel(e0[c], e1[c], four ? 2 : 1, 1, four) << (8 * c);
+    if (four) p[3] |= (uint32_t)palette_channel(e0[c], e1[c], 1, 2, true) << (8 * c);  // else black
+  }
+  uint32_t* out = const_cast<uint32_t*>(M.tex[R.level]) + 16 * (int64_t)M.mip_off[R.level][m] +
+                  (int64_t)(4 * by) * V.w + 4 * bx;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    uint32_t t[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const uint32_t i = bits >> (2 * (4 * r + x));
+      const uint32_t lo = (i & 1u) ? p[1] : p[0], hi = (i & 1u) ? p[3] : p[2];
+      t[x] = (i & 2u) ? hi : lo;
+    }
+    *reinterpret_cast<uint4*>(out + (int64_t)r * V.w) = make_uint4(t[0], t[1], t[2], t[3]);
+  }
+}
+
 }  // namespace nbtc
 
 using namespace nbtc;
@@ -203,6 +260,9 @@ struct nbtc_batch {
   WorkChunk* fchunks = nullptr;
   int* fcounter = nullptr;
   size_t plist_ints = 0;
+  uint32_t* texels = nullptr;  // decoded texels of every material's levels and mips (NULL: BC1 at the taps)
+  TexelRun* truns = nullptr;
+  int ntruns = 0;
   // tuned configuration and graphs
   int W = 3, Wf = 3, chunk = 32, tw = 16, th = 8;  // W: decode warpgroups, Wf: render warpgroups
   int ta = 0, taf = 0;  // A operands in TMEM (4 warpgroups x 1 slot) for the decode / the frame
@@ -295,6 +355,10 @@ static nbtc_status enqueue_render(nbtc_context* ctx, nbtc_batch* B, cudaStream_t
   const int blocks = (F.tiles + 7) / 8;
   k_frame_classify<<<blocks, 256, F.nmat * sizeof(int), s>>>(F);
   if ((st = cuda_check(cudaGetLastError(), "launch k_frame_classify"))) return st;
+  if (B->ntruns) {
+    k_frame_texels<<<B->ntruns, kTexelRun, 0, s>>>(B->truns, B->mats_dev, F);
+    if ((st = cuda_check(cudaGetLastError(), "launch k_frame_texels"))) return st;
+  }
   k_frame_scan<<<1, 256, (F.nmat + 1) * sizeof(int), s>>>(F);
   if ((st = cuda_check(cudaGetLastError(), "launch k_frame_scan"))) return st;
   k_frame_bin<<<blocks, 256, 0, s>>>(F);
@@ -310,6 +374,7 @@ static nbtc_status enqueue_render(nbtc_context* ctx, nbtc_batch* B, cudaStream_t
   p.flod = B->frame.lod;
   p.fduv = B->frame.duv;
   p.max_aniso = B->frame.duv ? B->frame.max_aniso : 1;
+  p.ftex = B->texels != nullptr;
   p.fshade = B->frame.shaded;
   p.light = make_light(B->frame);
   p.fout = static_cast<uint16_t*>(B->frame.out);
@@ -385,6 +450,21 @@ static nbtc_status capture(nbtc_context* ctx, nbtc_batch* B, bool render, cudaGr
   return st;
 }
 
+// Whether a frame of `pixels` decodes its materials' latents (`texels` of them, all
+// levels and mips) once per frame instead of at its taps.  Decoding a texel and
+// keeping it in HBM costs 4 bytes of writes, a tap of a BC1 texel ~45 instructions
+// more than one of a decoded texel, at 32 taps a pixel and more: up to 16 texels
+// a pixel (64 bytes; 0.5 GB for a 3840 x 2160 frame) decoding first is far
+// ahead, and the bound keeps a small frame of very many large materials from
+// holding, and filling, gigabytes.  The decoded taps wrap a texel index by one
+// period, so shifts beyond half a texel stay with the general path.
+static bool frame_texels_rule(const std::vector<MatDev>& md, int64_t texels, int64_t pixels) {
+  for (const MatDev& d : md)
+    for (int k = 0; k < 4; ++k)
+      if (!(std::fabs(d.d.lv[k].shift) <= 0.5f) || d.mip_off[k][NBTC_MAX_MIPS - 1] > (1 << 26)) return false;
+  return texels <= 16 * pixels;
+}
+
 static void free_plan(nbtc_batch* B) {
   if (!B) return;
   cudaSetDevice(B->device);
@@ -398,6 +478,8 @@ static void free_plan(nbtc_batch* B) {
   cudaFree(B->dnchunks);
   cudaFree(B->dcounter);
   cudaFree(B->frame_block);
+  cudaFree(B->texels);
+  cudaFree(B->truns);
   cudaFree(B->fchunks);
   cudaFree(B->fcounter);
   delete B;
@@ -510,6 +592,33 @@ nbtc_status nbtc_batch_create(nbtc_context* ctx, const nbtc_batch_material* mats
         w = std::max(4, w / 2);
         h = std::max(4, h / 2);
       }
+    }
+  }
+  // ---- frame: decoded texels of every level and its mips, and the runs of blocks that fill them
+  if (frame) {
+    int64_t texels = 0;
+    auto level_blocks = [&](int m, int k) {
+      const MatDev& d = md[m];
+      const nbtc_level& Lv = mats[m].latents.levels[k];
+      const int last = d.mips[k] - 1;
+      return d.mip_off[k][last] + (std::max(4, Lv.width >> last) / 4) * (std::max(4, Lv.height >> last) / 4);
+    };
+    for (int m = 0; m < count; ++m)
+      for (int k = 0; k < 4; ++k) texels += 16 * (int64_t)level_blocks(m, k);
+    if (frame_texels_rule(md, texels, (int64_t)frame->width * frame->height)) {
+      NBTC_TRY(cuda_check(cudaMalloc(&B->texels, (size_t)texels * sizeof(uint32_t)), "frame texels"));
+      std::vector<TexelRun> runs;
+      int64_t at = 0;
+      for (int m = 0; m < count; ++m)
+        for (int k = 0; k < 4; ++k) {
+          const int n = level_blocks(m, k);
+          md[m].tex[k] = B->texels + at;
+          for (int i = 0; i < n; i += kTexelRun) runs.push_back(TexelRun{m, k, i, std::min(kTexelRun, n - i)});
+          at += 16 * (int64_t)n;
+        }
+      B->ntruns = (int)runs.size();
+      NBTC_TRY(cuda_check(cudaMalloc(&B->truns, sizeof(TexelRun) * runs.size()), "texel runs"));
+      NBTC_TRY(upload(B->truns, runs.data(), sizeof(TexelRun) * runs.size(), s));
     }
   }
   NBTC_TRY(cuda_check(cudaMalloc(&B->mats_dev, sizeof(MatDev) * count), "plan table"));

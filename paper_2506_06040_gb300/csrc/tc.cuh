@@ -116,6 +116,7 @@ struct TcArgs {
   const float* flod;       // frame: per-pixel lod (log2 of the uv footprint + bias), or the bias with fduv
   const float* fduv;       // frame: per-pixel uv derivatives (anisotropic filter) or NULL
   int max_aniso;           // frame: probe cap of the anisotropic filter
+  int ftex;                // frame: taps read the materials' decoded texels (MatDev::tex)
   float* fshade;           // frame: lighting pass output (FP32 RGBA per pixel) or NULL
   LightDev light;          // frame: lighting constants
   uint16_t* fout;          // frame: per-pixel output (nout FP16)

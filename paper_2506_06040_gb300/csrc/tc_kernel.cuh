@@ -449,11 +449,16 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           const int64_t px = frame_pixel(p, work.c, T, gt);
           const int64_t pq = px < 0 ? 0 : px;
           const float2 uv = __ldg(reinterpret_cast<const float2*>(p.fuv) + pq);
-          if (p.fduv)
-            aniso_features(work.m, uv.x, uv.y, __ldg(reinterpret_cast<const float4*>(p.fduv) + pq), __ldg(p.flod + pq),
-                           p.max_aniso, f);
-          else
-            trilinear_features(work.m, uv.x, uv.y, __ldg(p.flod + pq), f);
+          const float lod = __ldg(p.flod + pq);
+          if (p.fduv) {
+            const float4 duv = __ldg(reinterpret_cast<const float4*>(p.fduv) + pq);
+            if (p.ftex) aniso_features<true>(work.m, uv.x, uv.y, duv, lod, p.max_aniso, f);
+            else aniso_features<false>(work.m, uv.x, uv.y, duv, lod, p.max_aniso, f);
+          } else if (p.ftex) {
+            trilinear_texels(work.m, uv.x, uv.y, lod, f);
+          } else {
+            trilinear_features(work.m, uv.x, uv.y, lod, f);
+          }
         }
       };
       // TA: a tile's A0 row as it goes into TMEM (8 columns; split FP16: hi in

@@ -139,6 +139,43 @@ def test_frame_anisotropic_filter_all_pixels(nb, ctx, max_aniso):
     plan.close()
 
 
+@pytest.mark.parametrize("aniso", [False, True])
+@pytest.mark.parametrize("address", ["wrap", "clamp"])
+@pytest.mark.parametrize("size,side", [((128, 64), 1024), ((144, 72), 256), ((512, 256), 1024)])
+def test_frame_decoded_texels_and_bc1_taps(nb, ctx, size, side, address, aniso):
+    """Both ways a frame reads its latents, every pixel against the oracle: up to 16
+    latent texels a pixel every texel is decoded once per frame, beyond that (the
+    small frame of large materials) BC1 is decoded at the taps.  Clamped and wrapped
+    coordinates outside [0, 1), and a pixel range without a material."""
+    w, h = size
+    bw = synth.batch_workload(num_materials=3, frame_w=w, frame_h=h, smin=side, smax=side, seed=91)
+    texels = sum(sum(16 * len(b) for lv in m.levels for b in lv.blocks) for m in bw.materials)
+    assert (texels <= 16 * w * h) == (w > 128)
+    for m in bw.materials:
+        m.address = address
+    bw.mat_id[: h // 8] = -1
+    bw.uv = (bw.uv - np.float32(1.25)).astype(np.float32)
+    fr = _frame_tensors(bw)
+    if aniso:
+        fr["duv"] = torch.from_numpy(np.ascontiguousarray(bw.duv)).cuda()
+        fr["max_aniso"], fr["lod"] = 16, torch.from_numpy(np.ascontiguousarray(bw.lod_bias)).cuda()
+    plan = nb.Batch(ctx, [nb.Material.from_synth(m) for m in bw.materials], None, fr, autotune=False)
+    plan.render()
+    ctx.sync()
+    if not aniso:
+        _frame_check(bw, fr["out"], np.arange(w * h))
+    else:
+        got = fr["out"].view(-1, 9).float().cpu().numpy().astype(np.float64)
+        ids = bw.mat_id.reshape(-1)
+        for m in np.unique(ids[ids >= 0]):
+            sel, mat = ids == m, bw.materials[m]
+            mips = [oracle.frame.level_mips_rgb(lv) for lv in mat.levels]
+            x = oracle.frame.aniso_features(mat, mips, bw.uv.reshape(-1, 2)[sel], bw.duv.reshape(-1, 4)[sel],
+                                            bw.lod_bias.reshape(-1)[sel], 16)
+            tp.check_interval(got[sel], mat, x, "fp16", sigma_x=SIGMA_ANISO, what=f"aniso material {m}")
+    plan.close()
+
+
 def test_frame_lighting_pass(nb, ctx):
     """The fused lighting pass against the oracle's shading of the same FP16
     G-buffer values the kernel produced.  FP32 vs FP64: the GGX term is the only
