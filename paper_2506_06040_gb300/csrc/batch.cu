@@ -262,6 +262,8 @@ struct nbtc_batch {
   size_t plist_ints = 0;
   uint32_t* texels = nullptr;  // decoded texels of every material's levels and mips (NULL: BC1 at the taps)
   TexelRun* truns = nullptr;
+  FrameLevel* flevels = nullptr;  // the feature pass's view of them
+  uint2* ffeat = nullptr;         // per-pixel features of the frame, 24 bytes each
   int ntruns = 0;
   // tuned configuration and graphs
   int W = 3, Wf = 3, chunk = 32, tw = 16, th = 8;  // W: decode warpgroups, Wf: render warpgroups
@@ -363,6 +365,20 @@ static nbtc_status enqueue_render(nbtc_context* ctx, nbtc_batch* B, cudaStream_t
   if ((st = cuda_check(cudaGetLastError(), "launch k_frame_scan"))) return st;
   k_frame_bin<<<blocks, 256, 0, s>>>(F);
   if ((st = cuda_check(cudaGetLastError(), "launch k_frame_bin"))) return st;
+  FrameFeatArgs f;
+  f.mat_id = F.mat_id;
+  f.uv = B->frame.uv;
+  f.lod = B->frame.lod;
+  f.duv = B->frame.duv;
+  f.max_aniso = B->frame.duv ? B->frame.max_aniso : 1;
+  f.nmat = F.nmat;
+  f.pixels = (int64_t)F.w * F.h;
+  f.levels = B->flevels;
+  f.mats = B->mats_dev;
+  f.feat = B->ffeat;
+  f.status = ctx->status_dev;
+  f.plant = ctx->check_plant;
+  if ((st = launch_frame_features(f, s))) return st;
   TcArgs p = base_args(ctx, B);
   p.chunks = B->fchunks;
   p.nchunks_dev = F.nchunks;
@@ -370,11 +386,7 @@ static nbtc_status enqueue_render(nbtc_context* ctx, nbtc_batch* B, cudaStream_t
   p.ulist = F.ulist;
   p.plist = F.plist;
   p.fmat = B->frame.mat_id;
-  p.fuv = B->frame.uv;
-  p.flod = B->frame.lod;
-  p.fduv = B->frame.duv;
-  p.max_aniso = B->frame.duv ? B->frame.max_aniso : 1;
-  p.ftex = B->texels != nullptr;
+  p.ffeat = B->ffeat;
   p.fshade = B->frame.shaded;
   p.light = make_light(B->frame);
   p.fout = static_cast<uint16_t*>(B->frame.out);
@@ -480,6 +492,8 @@ static void free_plan(nbtc_batch* B) {
   cudaFree(B->frame_block);
   cudaFree(B->texels);
   cudaFree(B->truns);
+  cudaFree(B->flevels);
+  cudaFree(B->ffeat);
   cudaFree(B->fchunks);
   cudaFree(B->fcounter);
   delete B;
@@ -605,20 +619,34 @@ nbtc_status nbtc_batch_create(nbtc_context* ctx, const nbtc_batch_material* mats
     };
     for (int m = 0; m < count; ++m)
       for (int k = 0; k < 4; ++k) texels += 16 * (int64_t)level_blocks(m, k);
+    NBTC_TRY(cuda_check(cudaMalloc(&B->ffeat, (size_t)frame->width * frame->height * 3 * sizeof(uint2)), "frame features"));
     if (frame_texels_rule(md, texels, (int64_t)frame->width * frame->height)) {
       NBTC_TRY(cuda_check(cudaMalloc(&B->texels, (size_t)texels * sizeof(uint32_t)), "frame texels"));
       std::vector<TexelRun> runs;
+      std::vector<FrameLevel> levels((size_t)count * 4);
       int64_t at = 0;
       for (int m = 0; m < count; ++m)
         for (int k = 0; k < 4; ++k) {
           const int n = level_blocks(m, k);
           md[m].tex[k] = B->texels + at;
           for (int i = 0; i < n; i += kTexelRun) runs.push_back(TexelRun{m, k, i, std::min(kTexelRun, n - i)});
+          FrameLevel& fl = levels[(size_t)m * 4 + k];
+          memset(&fl, 0, sizeof(fl));
+          fl.base = md[m].tex[k];
+          fl.log2w = md[m].log2w[k];
+          fl.shift = md[m].d.lv[k].shift;
+          fl.last = (float)(md[m].mips[k] - 1);
+          fl.wrap = md[m].d.wrap;
+          for (int i = 0; i < md[m].mips[k]; ++i)
+            fl.mip[i] = FrameMip{16u * (uint32_t)md[m].mip_off[k][i], std::max(4, md[m].d.lv[k].w >> i),
+                                 std::max(4, md[m].d.lv[k].h >> i), 0};
           at += 16 * (int64_t)n;
         }
       B->ntruns = (int)runs.size();
       NBTC_TRY(cuda_check(cudaMalloc(&B->truns, sizeof(TexelRun) * runs.size()), "texel runs"));
       NBTC_TRY(upload(B->truns, runs.data(), sizeof(TexelRun) * runs.size(), s));
+      NBTC_TRY(cuda_check(cudaMalloc(&B->flevels, sizeof(FrameLevel) * levels.size()), "frame levels"));
+      NBTC_TRY(upload(B->flevels, levels.data(), sizeof(FrameLevel) * levels.size(), s));
     }
   }
   NBTC_TRY(cuda_check(cudaMalloc(&B->mats_dev, sizeof(MatDev) * count), "plan table"));

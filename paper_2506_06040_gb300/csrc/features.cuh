@@ -404,13 +404,6 @@ __device__ __forceinline__ void warp_strip_features(const DecodeArgs& a, int j, 
   }
 }
 
-// i / n1 correctly rounded for the probe counts (1 <= i < n1 <= 17), r = RN(1 / n1):
-// the correction step of gridcoord.h (checked for every pair on the host).
-__device__ __forceinline__ float probe_fraction(float i, float n1, float r) {
-  const float q = __fmul_rn(i, r);
-  return fmaf(fmaf(-q, n1, i), r, q);
-}
-
 // Per-material description used by the batched and frame decodes: the level
 // views of mip 0 (in `d`) plus every level's mip chain for trilinear sampling.
 struct MatDev {
@@ -434,175 +427,6 @@ __device__ __forceinline__ LevelView mip_view(const MatDev& M, int k, int m) {
   v.h = max(4, v.h >> m);
   v.wb = v.w / 4;
   return v;
-}
-
-// ---- trilinear sampling of decoded texels.  A frame tap that decodes its BC1
-// texel costs ~65 instructions (two endpoints widened, three palette channels
-// with a division, three conversions) and a pixel takes 32 taps (288 with the
-// anisotropic filter), against ~0.1 .. 1 latent texels per pixel in the mip chains
-// themselves: so the frame decodes every texel of its visible materials once
-// (k_frame_texels) and its taps read RGBA8 words, ~18 instructions each with
-// the bilinear blend.  Same texels, weights and FP32 blend order up to rounding.
-
-// Channel c of an RGBA8 word as 2^23 + value (one byte permute, exact).
-__device__ __forceinline__ float byte_magic(uint32_t t, int c) {
-  return __uint_as_float(__byte_perm(t, 0x4B000000u, 0x7440u + (uint32_t)c));
-}
-
-// One mip's decoded texels.
-struct TexelView {
-  const uint32_t* t;
-  int w, h;
-  float shift;
-#ifdef NBTC_CHECKED
-  int* status;
-  int32_t plant;
-#endif
-};
-
-__device__ __forceinline__ TexelView texel_view(const MatDev& M, int k, int m) {
-  TexelView v;
-  v.t = M.tex[k] + 16 * (int64_t)M.mip_off[k][m];
-  v.w = max(4, M.d.lv[k].w >> m);
-  v.h = max(4, M.d.lv[k].h >> m);
-  v.shift = M.d.lv[k].shift;
-#ifdef NBTC_CHECKED
-  v.status = M.d.lv[k].status;
-  v.plant = M.d.lv[k].plant;
-#endif
-  return v;
-}
-
-__device__ __forceinline__ uint32_t texel_at(const TexelView& T, int i) {
-#ifdef NBTC_CHECKED
-  int64_t c = (int64_t)i + T.plant;
-  NBTC_CHECK_INDEX(c, (int64_t)T.w * T.h, T.status);
-  i = (int)c;
-#endif
-  return __ldg(T.t + i);
-}
-
-// Bilinear sample in 0..255 units: the horizontal blends of both rows as packed
-// FP32 pairs, then the vertical one.
-__device__ __forceinline__ float3 sample_texels(const TexelView& T, float u, float v, bool wrap) {
-  int x0, x1, y0, y1;
-  float fx, fy;
-  axis_taps(u, T.w, T.shift, wrap, x0, x1, fx);
-  axis_taps(v, T.h, T.shift, wrap, y0, y1, fy);
-  const int r0 = y0 * T.w, r1 = y1 * T.w;
-  const uint32_t t00 = texel_at(T, r0 + x0), t10 = texel_at(T, r0 + x1);
-  const uint32_t t01 = texel_at(T, r1 + x0), t11 = texel_at(T, r1 + x1);
-  float c[3];
-#pragma unroll
-  for (int ch = 0; ch < 3; ++ch) {
-    const float2 a = make_float2(byte_magic(t00, ch), byte_magic(t01, ch));
-    const float2 b = make_float2(byte_magic(t10, ch), byte_magic(t11, ch));
-    const float2 d = __fadd2_rn(b, make_float2(-a.x, -a.y));                   // exact
-    const float2 z = __fadd2_rn(a, make_float2(-8388608.f, -8388608.f));       // exact
-    const float2 r = __ffma2_rn(make_float2(fx, fx), d, z);
-    c[ch] = fmaf(fy, r.y - r.x, r.x);
-  }
-  return make_float3(c[0], c[1], c[2]);
-}
-
-// The two mips and the blend of level k at lod `lam` (unclamped).
-struct MipPair {
-  int m0, m1;
-  float t;
-};
-__device__ __forceinline__ MipPair mip_pair(const MatDev& M, int k, float lam) {
-  lam = fminf(fmaxf(lam, 0.f), (float)(M.mips[k] - 1));
-  MipPair P;
-  P.m0 = (int)floorf(lam);
-  P.m1 = min(P.m0 + 1, M.mips[k] - 1);
-  P.t = lam - (float)P.m0;
-  return P;
-}
-
-// trilinear_features on decoded texels.
-__device__ __forceinline__ void trilinear_texels(const MatDev& M, float u, float v, float lod, float (&feat)[12]) {
-  const bool wrap = M.d.wrap;
-  const float s = 1.0f / 255.0f;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const MipPair P = mip_pair(M, k, lod + M.log2w[k]);
-    const float3 c0 = sample_texels(texel_view(M, k, P.m0), u, v, wrap);
-    const float3 c1 = sample_texels(texel_view(M, k, P.m1), u, v, wrap);
-    feat[3 * k + 0] = s * fmaf(P.t, c1.x - c0.x, c0.x);
-    feat[3 * k + 1] = s * fmaf(P.t, c1.y - c0.y, c0.y);
-    feat[3 * k + 2] = s * fmaf(P.t, c1.z - c0.z, c0.z);
-  }
-}
-
-// Features of one pixel of the frame: per level, lod_k = lod + log2(W_k)
-// clamped to the mip range, trilinear (bilinear in mips floor(lod_k) and the
-// next, blended by its fraction), the material's address mode.
-__device__ __forceinline__ void trilinear_features(const MatDev& M, float u, float v, float lod, float (&feat)[12]) {
-  const bool wrap = M.d.wrap;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float lam = fminf(fmaxf(lod + M.log2w[k], 0.f), (float)(M.mips[k] - 1));
-    const int m0 = (int)floorf(lam);
-    const int m1 = min(m0 + 1, M.mips[k] - 1);
-    const float t = lam - (float)m0;
-    const float3 c0 = sample_bilinear(mip_view(M, k, m0), u, v, wrap);
-    const float3 c1 = sample_bilinear(mip_view(M, k, m1), u, v, wrap);
-    feat[3 * k + 0] = fmaf(t, c1.x - c0.x, c0.x);
-    feat[3 * k + 1] = fmaf(t, c1.y - c0.y, c0.y);
-    feat[3 * k + 2] = fmaf(t, c1.z - c0.z, c0.z);
-  }
-}
-
-// Anisotropic latent filter of one frame pixel (the reference formulas of the
-// anisotropic-filtering extension, in texture-coordinate units -- the square
-// latents make Pmax / Pmin the same for every level): N = min(ceil(Pmax /
-// Pmin), max_aniso) trilinear probes at uv + (i / (N + 1) - 1/2) d along the
-// major-axis derivative d, each level at lod bias + log2(Pmax W_k / N),
-// averaged.  N is decided with correctly rounded FP32 operations in a fixed
-// order (no contraction), so any IEEE implementation decides it alike.  The
-// mip pair of a level is the same for all probes, so levels run outermost
-// (TEX: its decoded texels' views are formed once; otherwise BC1 at the taps).
-template <bool TEX>
-__device__ __forceinline__ void aniso_features(const MatDev& M, float u, float v, float4 d, float bias,
-                                               int max_aniso, float (&feat)[12]) {
-  const float px = __fsqrt_rn(__fadd_rn(__fmul_rn(d.x, d.x), __fmul_rn(d.y, d.y)));
-  const float py = __fsqrt_rn(__fadd_rn(__fmul_rn(d.z, d.z), __fmul_rn(d.w, d.w)));
-  const bool along_x = px >= py;
-  const float pmax = along_x ? px : py, pmin = along_x ? py : px;
-  int n = 1;
-  if (pmax > 0.f) n = pmin > 0.f ? (int)fminf(ceilf(__fdiv_rn(pmax, pmin)), (float)max_aniso) : max_aniso;
-  const float au = along_x ? d.x : d.z, av = along_x ? d.y : d.w;
-  const float base = bias + log2f(pmax / (float)n);  // -inf for a zero footprint: clamps to mip 0
-  const bool wrap = M.d.wrap;
-  const float n1 = (float)(n + 1), rn1 = 1.0f / n1;
-  const float inv = (TEX ? 1.0f / 255.0f : 1.0f) / (float)n;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const MipPair P = mip_pair(M, k, base + M.log2w[k]);
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-    auto probes = [&](auto&& sample0, auto&& sample1) {
-#pragma unroll 1
-      for (int i = 1; i <= n; ++i) {
-        const float off = probe_fraction((float)i, n1, rn1) - 0.5f;
-        const float uu = fmaf(off, au, u), vv = fmaf(off, av, v);
-        const float3 c0 = sample0(uu, vv), c1 = sample1(uu, vv);
-        a0 += fmaf(P.t, c1.x - c0.x, c0.x);
-        a1 += fmaf(P.t, c1.y - c0.y, c0.y);
-        a2 += fmaf(P.t, c1.z - c0.z, c0.z);
-      }
-    };
-    if constexpr (TEX) {
-      const TexelView V0 = texel_view(M, k, P.m0), V1 = texel_view(M, k, P.m1);
-      probes([&](float uu, float vv) { return sample_texels(V0, uu, vv, wrap); },
-             [&](float uu, float vv) { return sample_texels(V1, uu, vv, wrap); });
-    } else {
-      probes([&](float uu, float vv) { return sample_bilinear(mip_view(M, k, P.m0), uu, vv, wrap); },
-             [&](float uu, float vv) { return sample_bilinear(mip_view(M, k, P.m1), uu, vv, wrap); });
-    }
-    feat[3 * k + 0] = a0 * inv;
-    feat[3 * k + 1] = a1 * inv;
-    feat[3 * k + 2] = a2 * inv;
-  }
 }
 
 // Features of one texel sampled on its own (any uv).

@@ -112,11 +112,7 @@ struct TcArgs {
   const int* ulist;        // frame: uniform screen tiles
   const int* plist;        // frame: packed pixel indices (128 per tile, -1 = none)
   const int* fmat;         // frame: per-pixel material id
-  const float* fuv;        // frame: per-pixel uv
-  const float* flod;       // frame: per-pixel lod (log2 of the uv footprint + bias), or the bias with fduv
-  const float* fduv;       // frame: per-pixel uv derivatives (anisotropic filter) or NULL
-  int max_aniso;           // frame: probe cap of the anisotropic filter
-  int ftex;                // frame: taps read the materials' decoded texels (MatDev::tex)
+  const uint2* ffeat;      // frame: per-pixel features, 12 FP16 (k_frame_features)
   float* fshade;           // frame: lighting pass output (FP32 RGBA per pixel) or NULL
   LightDev light;          // frame: lighting constants
   uint16_t* fout;          // frame: per-pixel output (nout FP16)
@@ -134,6 +130,38 @@ struct TcWork {
 };
 
 
+
+// One level of one material as the frame's feature pass reads it: decoded texels
+// of all mips from `base`, mip m at texel off[m].
+struct FrameMip {
+  uint32_t off;
+  int32_t w, h, pad;
+};
+struct FrameLevel {
+  const uint32_t* base;
+  float log2w, shift;
+  float last;    // num_mips - 1
+  int32_t wrap;
+  int32_t pad[2];
+  FrameMip mip[NBTC_MAX_MIPS];
+};
+
+// Arguments of the frame's feature pass.
+struct FrameFeatArgs {
+  const int* mat_id;
+  const float* uv;
+  const float* lod;           // lod, or the mip bias with duv
+  const float* duv;           // NULL: trilinear
+  int max_aniso;
+  int nmat;
+  int64_t pixels;
+  const FrameLevel* levels;   // [nmat][4], or NULL: BC1 decoded at the taps
+  const MatDev* mats;
+  uint2* feat;                // [pixels][3]
+  int* status;                // checked build
+  int plant;
+};
+nbtc_status launch_frame_features(const FrameFeatArgs& a, cudaStream_t s);
 
 struct TcArgs;
 // Launches the decode kernel (any mode) with W warpgroups of `slots` tile

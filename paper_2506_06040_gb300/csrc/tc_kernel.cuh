@@ -431,34 +431,17 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
       strip_reset(cache);
       uint32_t next_a0[16];  // TA: the next tile's A0, computed during the output layer's MMAs
 
-      // features of tile T (chunk numbering) into slot s's A0, then A-ready
-      // the 12 features of this thread's texel (or frame pixel) of tile T
+      // the 12 features of this thread's texel of tile T (full decode)
       auto tile_features = [&](int64_t T, float (&f)[12]) {
-        if (MODE == kModeSingle || grid_chunk) {
-          if (footprint) {
-            // tile number = column block x H + row; each warp decodes its own
-            // 32 texels' latent columns and shares them by shuffles
-            const uint32_t t = (uint32_t)(work.c.first + T), H = (uint32_t)D.grid_h;
-            const uint32_t cb = fastdiv(t, hdiv);
-            warp_strip_features(D, (int)(t - cb * H), (int)cb * kTile + 32 * wq, lane, cache, f);
-          } else {
-            const int64_t tex = (work.c.first + T) * kTile + gt;
-            direct_features(D, tex < D.n ? tex : D.n - 1, f);
-          }
+        if (footprint) {
+          // tile number = column block x H + row; each warp decodes its own
+          // 32 texels' latent columns and shares them by shuffles
+          const uint32_t t = (uint32_t)(work.c.first + T), H = (uint32_t)D.grid_h;
+          const uint32_t cb = fastdiv(t, hdiv);
+          warp_strip_features(D, (int)(t - cb * H), (int)cb * kTile + 32 * wq, lane, cache, f);
         } else {
-          const int64_t px = frame_pixel(p, work.c, T, gt);
-          const int64_t pq = px < 0 ? 0 : px;
-          const float2 uv = __ldg(reinterpret_cast<const float2*>(p.fuv) + pq);
-          const float lod = __ldg(p.flod + pq);
-          if (p.fduv) {
-            const float4 duv = __ldg(reinterpret_cast<const float4*>(p.fduv) + pq);
-            if (p.ftex) aniso_features<true>(work.m, uv.x, uv.y, duv, lod, p.max_aniso, f);
-            else aniso_features<false>(work.m, uv.x, uv.y, duv, lod, p.max_aniso, f);
-          } else if (p.ftex) {
-            trilinear_texels(work.m, uv.x, uv.y, lod, f);
-          } else {
-            trilinear_features(work.m, uv.x, uv.y, lod, f);
-          }
+          const int64_t tex = (work.c.first + T) * kTile + gt;
+          direct_features(D, tex < D.n ? tex : D.n - 1, f);
         }
       };
       // TA: a tile's A0 row as it goes into TMEM (8 columns; split FP16: hi in
@@ -494,6 +477,26 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           av[7] = 0u;
         }
       };
+      // the packed A0 row of this thread's row of tile T: from the features of its
+      // texel, or (frame chunks, FP16 only) the row the feature pass left for its pixel
+      auto tile_row = [&](int64_t T, uint32_t (&av)[16]) {
+        if (MODE == kModeSingle || grid_chunk) {
+          float f[12];
+          tile_features(T, f);
+          pack_a0(f, av);
+        } else {
+          const int64_t px = frame_pixel(p, work.c, T, gt);
+          const uint2* r = p.ffeat + 3 * (px < 0 ? 0 : px);
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            const uint2 q = __ldg(r + i);
+            av[2 * i] = q.x;
+            av[2 * i + 1] = q.y;
+          }
+          av[6] = 0x3C00u;  // k = 12: 1.0 for the bias
+          av[7] = 0u;
+        }
+      };
       auto store_a0 = [&](int s, const uint32_t (&av)[16]) {
         const int q = wg * kSlots + s;
         const uint32_t ta = tmem_base + a_col(q) + lane_off;  // the slot's A (hi) columns
@@ -509,19 +512,23 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
       auto start_tile = [&](int s, int64_t T) {
         const int q = wg * kSlots + s;
         const uint32_t a0 = sbase + S.slots + q * S.slot + S.a0;
+        if constexpr (TA || FORM == kF16) {
+          uint32_t av[16];
+          tile_row(T, av);
+          if constexpr (TA) {
+            store_a0(s, av);
+            return;
+          }
+          sts128(a0 + off_interleave(gt, 0), av[0], av[1], av[2], av[3]);
+          sts128(a0 + off_interleave(gt, 16), av[4], av[5], av[6], av[7]);
+          fence_proxy_async_smem();
+          __syncwarp();
+          named_bar_arrive(bar_a(q), kTile + 32);
+          return;
+        }
         float f[12];
         tile_features(T, f);
-        if constexpr (TA) {
-          uint32_t av[16];
-          pack_a0(f, av);
-          store_a0(s, av);
-          return;
-        } else if constexpr (FORM == kF16) {
-          sts128(a0 + off_interleave(gt, 0), cvt_f16x2(f[0], f[1]), cvt_f16x2(f[2], f[3]), cvt_f16x2(f[4], f[5]),
-                 cvt_f16x2(f[6], f[7]));
-          sts128(a0 + off_interleave(gt, 16), cvt_f16x2(f[8], f[9]), cvt_f16x2(f[10], f[11]),
-                 0x3C00u /* k = 12: 1.0 for the bias */, 0u);
-        } else if constexpr (F16S) {
+        if constexpr (F16S) {
           uint32_t h[6], r[6];
 #pragma unroll
           for (int i = 0; i < 6; ++i) split_f16x2(f[2 * i], f[2 * i + 1], h[i], r[i]);
@@ -818,11 +825,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
               if constexpr (TA) {
                 // the next tile's features while the output layer's MMAs run
                 // (stored into TMEM once those have read this tile's A)
-                if (l == NHID - 1 && base + s + kSlots < g_end) {
-                  float f[12];
-                  tile_features(base + s + kSlots, f);
-                  pack_a0(f, next_a0);
-                }
+                if (l == NHID - 1 && base + s + kSlots < g_end) tile_row(base + s + kSlots, next_a0);
               }
             } else {
               const bool more = base + s + kSlots < g_end;
