@@ -10,16 +10,16 @@
 //
 // Frame: pass A (k_frame_classify) marks each 128-pixel tile uniform or mixed
 // and counts, per material, uniform tiles and valid pixels of mixed tiles
-// (per-CTA shared-memory histograms, then one global atomic per material --
-// the paper suggests shared-memory atomics for this, Sec. 6); k_frame_scan
-// turns the counts into slot offsets (an exclusive prefix sum; Algorithm 1
-// reads these offsets but does not say how they are made) and into the chunk
-// list; pass B (k_frame_bin) appends uniform tiles to their material's list and
-// packs mixed-tile pixels into their material's 128-slot tiles (warp-aggregated
-// atomics: one atomic per material present in a warp).  Then the decode kernel
-// runs over those chunks.  Between the passes k_frame_texels decodes the visible
-// materials' latent texels once (see the rule at frame_texels_rule).  All the
-// launches are captured in one CUDA graph.
+// (per-CTA shared-memory histograms, then one global atomic per CTA and material
+// -- the paper suggests shared-memory atomics for this, Sec. 6 -- whose old
+// value is the CTA's place in the material's list); k_frame_scan turns the counts
+// into slot offsets (an exclusive prefix sum; Algorithm 1 reads these offsets but
+// does not say how they are made) and into the chunk list, while its other CTAs
+// decode the visible materials' latent texels (see frame_texels_rule); pass B
+// (k_frame_bin) appends uniform tiles to their material's list and packs
+// mixed-tile pixels into their material's 128-slot tiles.  k_frame_features
+// (frame_features.cu) leaves every pixel's features, and the decode kernel runs
+// over the chunks.  All the launches are captured in one CUDA graph.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -34,6 +34,7 @@ namespace nbtc {
 
 constexpr int kMaxMaterials = 1024;
 constexpr int kTileK = 128;  // pixels per classification tile
+constexpr int kClassifyCtas = 8 * 152;  // runs of tiles of the classification: 8 CTAs on each SM
 
 enum TileKind { kTileEmpty = 0, kTileUniform = 1, kTileMixed = 2 };
 
@@ -45,16 +46,20 @@ struct FrameDev {
   int* tmat;
   int* ucount;   // uniform tiles per material
   int* pcount;   // valid pixels of mixed tiles per material
-  int* ucur;
-  int* pcur;
+  int* ubase;    // [ctas][nmat] place of each CTA's uniform tiles in its material's list
+  int* pbase;    // [ctas][nmat] the same for the pixels of mixed tiles
   int* uoff;     // first slot in ulist
   int* poff;     // first packed tile
   int* ulist;
   int* plist;
   WorkChunk* chunks;
   int* nchunks;
+  int* counter;  // next chunk of the decode kernel (zeroed by the scan)
   int chunk_cap;
-  int chunk_tiles;
+  int decode_ctas;  // CTAs of the decode kernel
+  int ctas;         // CTAs of the classification and the binning, each with a run of tiles
+  int per_cta;      // tiles of a run
+  int ids16;        // mat_id may be read four pixels at a time
   int* stats;    // [uniform tiles, mixed tiles, packed tiles]
   int64_t ulist_cap, plist_cap;  // slots of ulist and plist (bounds of the checked build)
   int* status;                   // context status word (checked build)
@@ -67,20 +72,42 @@ __device__ __forceinline__ int tile_pixel(const FrameDev& F, int t, int j) {
   return (ty * F.th + r) * F.w + tx * F.tw + (j - r * F.tw);
 }
 
-// Pass A: one warp per tile, 4 pixels per lane.
-__global__ void k_frame_classify(FrameDev F) {
-  extern __shared__ int hist[];  // [nmat] mixed-tile pixel counts of this CTA
-  for (int m = threadIdx.x; m < F.nmat; m += blockDim.x) hist[m] = 0;
+// Material ids of the four pixels px .. px + 3 (one row of a tile; tile widths are
+// multiples of 4).  Ids past the table decode as "no material".
+__device__ __forceinline__ void tile_ids(const FrameDev& F, int px, int (&ids)[4]) {
+  if (F.ids16) {
+    const int4 q = __ldg(reinterpret_cast<const int4*>(F.mat_id + px));
+    ids[0] = q.x;
+    ids[1] = q.y;
+    ids[2] = q.z;
+    ids[3] = q.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ids[i] = __ldg(F.mat_id + px + i);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (ids[i] < 0 || ids[i] >= F.nmat) ids[i] = -1;
+}
+
+// Pass A: one warp per tile, 4 pixels per lane; a CTA takes a run of tiles and
+// touches global memory with one atomic per material it met (one per tile had
+// made it a queue at two addresses: 71 us for 65k tiles, 14 us now).
+__global__ void __launch_bounds__(256) k_frame_classify(FrameDev F) {
+  extern __shared__ int hist[];  // [nmat] uniform tiles, [nmat] pixels of mixed tiles, [2] tiles of each kind
+  int* hu = hist;
+  int* hp = hist + F.nmat;
+  int* hk = hist + 2 * F.nmat;
+  for (int m = threadIdx.x; m < 2 * F.nmat + 2; m += blockDim.x) hist[m] = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  if (t < F.tiles) {
+  const int first = blockIdx.x * F.per_cta, last = min(first + F.per_cta, F.tiles);
+  for (int t = first + threadIdx.x / 32; t < last; t += blockDim.x / 32) {
     int ids[4];
+    tile_ids(F, tile_pixel(F, t, lane * 4), ids);
     int cnt = 0, mn = 0x7fffffff, mx = -1;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      ids[i] = __ldg(F.mat_id + tile_pixel(F, t, lane * 4 + i));
-      if (ids[i] >= F.nmat) ids[i] = -1;  // out-of-range ids decode as "no material"
       if (ids[i] >= 0) {
         ++cnt;
         mn = min(mn, ids[i]);
@@ -94,87 +121,149 @@ __global__ void k_frame_classify(FrameDev F) {
     if (lane == 0) {
       F.tkind[t] = kind;
       F.tmat[t] = kind == kTileUniform ? mn : -1;
-      if (kind == kTileUniform) atomicAdd(F.ucount + mn, 1);
-      if (kind == kTileUniform) atomicAdd(F.stats + 0, 1);
-      if (kind == kTileMixed) atomicAdd(F.stats + 1, 1);
+      if (kind == kTileUniform) {
+        atomicAdd_block(hu + mn, 1);
+        atomicAdd_block(hk + 0, 1);
+      }
+      if (kind == kTileMixed) atomicAdd_block(hk + 1, 1);
     }
     if (kind == kTileMixed) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        if (ids[i] >= 0) atomicAdd_block(hist + ids[i], 1);
+        if (ids[i] >= 0) atomicAdd_block(hp + ids[i], 1);
     }
-  }
-  __syncthreads();
-  for (int m = threadIdx.x; m < F.nmat; m += blockDim.x)
-    if (hist[m]) atomicAdd(F.pcount + m, hist[m]);
-}
-
-// Offsets (exclusive scans) and the chunk list: per material its uniform-tile
-// chunks, then its packed-tile chunks.  One CTA.
-__global__ void k_frame_scan(FrameDev F) {
-  extern __shared__ int coff[];  // [nmat + 1] chunk offsets
-  if (threadIdx.x == 0) {
-    int su = 0, sp = 0, sc = 0;
-    for (int m = 0; m < F.nmat; ++m) {
-      const int U = F.ucount[m];
-      const int P = (F.pcount[m] + kTileK - 1) / kTileK;
-      F.uoff[m] = su;
-      F.poff[m] = sp;
-      coff[m] = sc;
-      su += U;
-      sp += P;
-      sc += (U + F.chunk_tiles - 1) / F.chunk_tiles + (P + F.chunk_tiles - 1) / F.chunk_tiles;
-    }
-    coff[F.nmat] = sc;
-    *F.nchunks = min(sc, F.chunk_cap);
-    F.stats[2] = sp;
   }
   __syncthreads();
   for (int m = threadIdx.x; m < F.nmat; m += blockDim.x) {
-    F.ucur[m] = 0;
-    F.pcur[m] = 0;
-    int c = coff[m];
-    const int U = F.ucount[m], P = (F.pcount[m] + kTileK - 1) / kTileK;
-    for (int i = 0; i < U; i += F.chunk_tiles, ++c)
-      if (c < F.chunk_cap) F.chunks[c] = WorkChunk{m, kChunkUniform, (int64_t)F.uoff[m] + i, min(F.chunk_tiles, U - i), 0};
-    for (int i = 0; i < P; i += F.chunk_tiles, ++c)
-      if (c < F.chunk_cap) F.chunks[c] = WorkChunk{m, kChunkPacked, (int64_t)F.poff[m] + i, min(F.chunk_tiles, P - i), 0};
+    if (hu[m]) F.ubase[(size_t)blockIdx.x * F.nmat + m] = atomicAdd(F.ucount + m, hu[m]);
+    if (hp[m]) F.pbase[(size_t)blockIdx.x * F.nmat + m] = atomicAdd(F.pcount + m, hp[m]);
+  }
+  if (threadIdx.x < 2 && hk[threadIdx.x]) atomicAdd(F.stats + threadIdx.x, hk[threadIdx.x]);
+}
+
+// Exclusive prefix sum of one value per thread over a 256-thread CTA; `total`
+// receives the sum.
+__device__ __forceinline__ int block_scan(int x, int& total, int* warp_sums) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int incl = x;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += y;
+  }
+  __syncthreads();  // the previous scan's sums have been read
+  if (lane == 31) warp_sums[warp] = incl;
+  __syncthreads();
+  int before = 0, sum = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    if (w < warp) before += warp_sums[w];
+    sum += warp_sums[w];
+  }
+  total = sum;
+  return before + incl - x;
+}
+
+// Offsets (exclusive scans) and the chunk list: per material its uniform-tile
+// chunks, then its packed-tile chunks.  One 256-thread CTA, `coff` [nmat + 1].
+// Every tile costs the decode kernel the same, and a chunk costs it a
+// reload of the MLP (~2 us), so chunks are a quarter of a CTA's share of the frame.
+__device__ void frame_scan(const FrameDev& F, int* coff, int* warp_sums) {
+  const int t = threadIdx.x;
+  int tiles = 0;
+  for (int m = t; m < F.nmat; m += blockDim.x) tiles += F.ucount[m] + (F.pcount[m] + kTileK - 1) / kTileK;
+  int all = 0;
+  block_scan(tiles, all, warp_sums);
+  const int chunk = max(16, (all + 4 * F.decode_ctas - 1) / (4 * F.decode_ctas));
+  int su = 0, sp = 0, sc = 0;
+  for (int m0 = 0; m0 < F.nmat; m0 += (int)blockDim.x) {
+    const int m = m0 + t;
+    const int U = m < F.nmat ? F.ucount[m] : 0;
+    const int px = m < F.nmat ? F.pcount[m] : 0;
+    const int P = (px + kTileK - 1) / kTileK;
+    const int C = (U + chunk - 1) / chunk + (P + chunk - 1) / chunk;
+    int tu, tp, tc;
+    const int u = su + block_scan(U, tu, warp_sums), q = sp + block_scan(P, tp, warp_sums),
+              c = sc + block_scan(C, tc, warp_sums);
+    if (m < F.nmat) {
+      F.uoff[m] = u;
+      F.poff[m] = q;
+      coff[m] = c;
+      for (int i = px; i < P * kTileK; ++i) F.plist[(int64_t)q * kTileK + i] = -1;  // the last packed tile's free slots
+    }
+    su += tu;
+    sp += tp;
+    sc += tc;
+  }
+  if (t == 0) {
+    coff[F.nmat] = sc;
+    *F.nchunks = min(sc, F.chunk_cap);
+    *F.counter = 0;
+    F.stats[2] = sp;
+  }
+  __syncthreads();
+  for (int c = t; c < min(sc, F.chunk_cap); c += blockDim.x) {
+    int lo = 0, hi = F.nmat - 1;  // the material whose chunks hold c: the last m with coff[m] <= c
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (coff[mid] <= c) lo = mid;
+      else hi = mid - 1;
+    }
+    const int m = lo, U = F.ucount[m], P = (F.pcount[m] + kTileK - 1) / kTileK;
+    const int nu = (U + chunk - 1) / chunk;
+    int i = c - coff[m];
+    if (i < nu) {
+      i *= chunk;
+      F.chunks[c] = WorkChunk{m, kChunkUniform, (int64_t)F.uoff[m] + i, min(chunk, U - i), 0};
+    } else {
+      i = (i - nu) * chunk;
+      F.chunks[c] = WorkChunk{m, kChunkPacked, (int64_t)F.poff[m] + i, min(chunk, P - i), 0};
+    }
   }
 }
 
-// Pass B: uniform tiles -> their material's list; mixed-tile pixels -> packed
-// slots of their material (one atomic per material present in the warp).
-__global__ void k_frame_bin(FrameDev F) {
-  const int lane = threadIdx.x & 31;
-  const int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  if (t >= F.tiles) return;
-  const int kind = F.tkind[t];
-  if (kind == kTileUniform) {
-    if (lane == 0) {
-      const int m = F.tmat[t];
-      const int pos = atomicAdd(F.ucur + m, 1);
-      int64_t slot = (int64_t)F.uoff[m] + pos;
-      NBTC_CHECK_INDEX(slot, F.ulist_cap, F.status);
-      F.ulist[slot] = t;
-    }
-    return;
+// Pass B, over the classification's runs of tiles: uniform tiles -> their
+// material's list; mixed-tile pixels -> packed slots of their material.  The
+// run's places were taken in pass A, so the cursors are shared-memory ones
+// (one atomic per material present in a warp).
+__global__ void __launch_bounds__(256) k_frame_bin(FrameDev F) {
+  extern __shared__ int cur[];  // [nmat] next slot in ulist, [nmat] next slot in plist
+  int* cu = cur;
+  int* cp = cur + F.nmat;
+  for (int m = threadIdx.x; m < F.nmat; m += blockDim.x) {  // places of materials the run does not hold are not used
+    cu[m] = F.uoff[m] + F.ubase[(size_t)blockIdx.x * F.nmat + m];
+    cp[m] = F.poff[m] * kTileK + F.pbase[(size_t)blockIdx.x * F.nmat + m];
   }
-  if (kind != kTileMixed) return;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
+  const int first = blockIdx.x * F.per_cta, last = min(first + F.per_cta, F.tiles);
+  for (int t = first + threadIdx.x / 32; t < last; t += blockDim.x / 32) {
+    const int kind = F.tkind[t];
+    if (kind == kTileUniform) {
+      if (lane == 0) {
+        int64_t slot = atomicAdd_block(cu + F.tmat[t], 1);
+        NBTC_CHECK_INDEX(slot, F.ulist_cap, F.status);
+        F.ulist[slot] = t;
+      }
+    } else if (kind == kTileMixed) {
+      const int px = tile_pixel(F, t, lane * 4);
+      int ids[4];
+      tile_ids(F, px, ids);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int px = tile_pixel(F, t, lane * 4 + i);
-    int id = __ldg(F.mat_id + px);
-    if (id >= F.nmat) id = -1;
-    const unsigned peers = __match_any_sync(0xffffffffu, id);
-    const int leader = __ffs(peers) - 1;
-    int base = 0;
-    if (id >= 0 && lane == leader) base = atomicAdd(F.pcur + id, __popc(peers));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (id >= 0) {
-      int64_t slot = (int64_t)F.poff[id] * kTileK + base + __popc(peers & lt);
-      NBTC_CHECK_INDEX(slot, F.plist_cap, F.status);
-      F.plist[slot] = px;
+      for (int i = 0; i < 4; ++i) {
+        const int id = ids[i];
+        const unsigned peers = __match_any_sync(0xffffffffu, id);
+        const int leader = __ffs(peers) - 1;
+        int base = 0;
+        if (id >= 0 && lane == leader) base = atomicAdd_block(cp + id, __popc(peers));
+        base = __shfl_sync(0xffffffffu, base, leader);
+        if (id >= 0) {
+          int64_t slot = (int64_t)base + __popc(peers & lt);
+          NBTC_CHECK_INDEX(slot, F.plist_cap, F.status);
+          F.plist[slot] = px + i;
+        }
+      }
     }
   }
 }
@@ -188,14 +277,21 @@ struct TexelRun {
 };
 constexpr int kTexelRun = 256;
 
-// One thread per block of a run: the block's four palette colours, then its 16
-// texels as RGBA8 words, four 16-byte row stores (neighbouring threads write
-// neighbouring 16 bytes of a row).  Materials without a pixel in this frame (the
-// counts of pass A) are left out.  Bound by its writes, 4 bytes per latent texel:
-// the 7.0 M texels of 64 materials up to 2048^2 take 9.9 us.
-__global__ void __launch_bounds__(kTexelRun) k_frame_texels(const TexelRun* __restrict__ runs, const MatDev* __restrict__ mats,
-                                                            FrameDev F) {
-  const TexelRun R = runs[blockIdx.x];
+// CTA 0: the offsets and the chunk list.  The others, one thread per block of a
+// run: the block's four palette colours, then its 16 texels as RGBA8 words, four
+// 16-byte row stores (neighbouring threads write neighbouring 16 bytes of a
+// row).  Materials without a pixel in this frame (the counts of pass A) are left
+// out.  Bound by its writes, 4 bytes per latent texel: the 7.0 M texels of 64
+// materials up to 2048^2 take 11 us, the scan included.
+__global__ void __launch_bounds__(kTexelRun) k_frame_scan(const TexelRun* __restrict__ runs,
+                                                          const MatDev* __restrict__ mats, FrameDev F) {
+  extern __shared__ int coff[];
+  __shared__ int warp_sums[8];
+  if (blockIdx.x == 0) {
+    frame_scan(F, coff, warp_sums);
+    return;
+  }
+  const TexelRun R = runs[blockIdx.x - 1];
   if (F.ucount[R.mat] + F.pcount[R.mat] == 0) return;
   if ((int)threadIdx.x >= R.count) return;
   const MatDev& M = mats[R.mat];
@@ -351,19 +447,11 @@ static nbtc_status enqueue_render(nbtc_context* ctx, nbtc_batch* B, cudaStream_t
   nbtc_status st;
   const size_t zero_ints = (size_t)2 * F.nmat + 3;  // ucount, pcount, stats are contiguous
   if ((st = cuda_check(cudaMemsetAsync(F.ucount, 0, zero_ints * sizeof(int), s), "reset frame counts"))) return st;
-  if ((st = cuda_check(cudaMemsetAsync(F.plist, 0xFF, B->plist_ints * sizeof(int), s), "reset packed slots")))
-    return st;
-  if ((st = cuda_check(cudaMemsetAsync(B->fcounter, 0, sizeof(int), s), "reset chunk counter"))) return st;
-  const int blocks = (F.tiles + 7) / 8;
-  k_frame_classify<<<blocks, 256, F.nmat * sizeof(int), s>>>(F);
+  k_frame_classify<<<F.ctas, 256, (2 * F.nmat + 2) * sizeof(int), s>>>(F);
   if ((st = cuda_check(cudaGetLastError(), "launch k_frame_classify"))) return st;
-  if (B->ntruns) {
-    k_frame_texels<<<B->ntruns, kTexelRun, 0, s>>>(B->truns, B->mats_dev, F);
-    if ((st = cuda_check(cudaGetLastError(), "launch k_frame_texels"))) return st;
-  }
-  k_frame_scan<<<1, 256, (F.nmat + 1) * sizeof(int), s>>>(F);
+  k_frame_scan<<<1 + B->ntruns, kTexelRun, (F.nmat + 1) * sizeof(int), s>>>(B->truns, B->mats_dev, F);
   if ((st = cuda_check(cudaGetLastError(), "launch k_frame_scan"))) return st;
-  k_frame_bin<<<blocks, 256, 0, s>>>(F);
+  k_frame_bin<<<F.ctas, 256, 2 * F.nmat * sizeof(int), s>>>(F);
   if ((st = cuda_check(cudaGetLastError(), "launch k_frame_bin"))) return st;
   FrameFeatArgs f;
   f.mat_id = F.mat_id;
@@ -391,6 +479,10 @@ static nbtc_status enqueue_render(nbtc_context* ctx, nbtc_batch* B, cudaStream_t
   p.light = make_light(B->frame);
   p.fout = static_cast<uint16_t*>(B->frame.out);
   p.frame_w = F.w;
+  {  // the pixels of a tile row of one warp are contiguous in the output: bulk copies of whole 16-byte pieces
+    const int seg = std::min(32, F.tw);
+    p.fseg = aligned(B->frame.out, 16) && (seg * B->nout * 2) % 16 == 0 && ((int64_t)F.tw * B->nout * 2) % 16 == 0 ? seg : 0;
+  }
   p.frame_pixels = (int64_t)F.w * F.h;
   p.tile_w = F.tw;
   p.tile_h = F.th;
@@ -406,6 +498,8 @@ static nbtc_status set_tile_shape(nbtc_batch* B, int tw, int th) {
   F.th = th;
   F.tiles_x = F.w / tw;
   F.tiles = F.tiles_x * (F.h / th);
+  F.per_cta = std::max(8, (F.tiles + kClassifyCtas - 1) / kClassifyCtas);  // at least a tile per warp
+  F.ctas = (F.tiles + F.per_cta - 1) / F.per_cta;
   B->tw = tw;
   B->th = th;
   return NBTC_OK;
@@ -666,19 +760,22 @@ nbtc_status nbtc_batch_create(nbtc_context* ctx, const nbtc_batch_material* mats
     F.w = frame->width;
     F.h = frame->height;
     F.nmat = count;
-    F.chunk_tiles = 16;
+    F.decode_ctas = ctx->sm_count;
+    F.ids16 = aligned(frame->mat_id, 16) && frame->width % 4 == 0;
     const int pixels = frame->width * frame->height;
     const int max_tiles = pixels / kTileK + 1;
     B->plist_ints = (size_t)(pixels / kTileK + count + 1) * kTileK;
-    const size_t ints = (size_t)2 * count + 3 /* counts + stats */ + 4 * (size_t)count /* cursors, offsets */ +
-                        2 * (size_t)max_tiles /* kind, mat */ + max_tiles /* ulist */ + B->plist_ints + 1;
+    const size_t runs = std::min(kClassifyCtas, max_tiles / 8 + 1);
+    const size_t ints = (size_t)2 * count + 3 /* counts + stats */ + 2 * (size_t)count /* offsets */ +
+                        2 * runs * count /* places */ + 2 * (size_t)max_tiles /* kind, mat */ + max_tiles /* ulist */ +
+                        B->plist_ints + 1;
     NBTC_TRY(cuda_check(cudaMalloc(&B->frame_block, ints * sizeof(int)), "frame buffers"));
     int* q = B->frame_block;
     F.ucount = q; q += count;
     F.pcount = q; q += count;
     F.stats = q; q += 3;
-    F.ucur = q; q += count;
-    F.pcur = q; q += count;
+    F.ubase = q; q += runs * count;
+    F.pbase = q; q += runs * count;
     F.uoff = q; q += count;
     F.poff = q; q += count;
     F.tkind = q; q += max_tiles;
@@ -693,6 +790,7 @@ nbtc_status nbtc_batch_create(nbtc_context* ctx, const nbtc_batch_material* mats
     NBTC_TRY(cuda_check(cudaMalloc(&B->fchunks, sizeof(WorkChunk) * F.chunk_cap), "frame chunks"));
     NBTC_TRY(cuda_check(cudaMalloc(&B->fcounter, sizeof(int)), "frame counter"));
     F.chunks = B->fchunks;
+    F.counter = B->fcounter;
     NBTC_TRY(set_tile_shape(B, 16, 8));
   }
   NBTC_TRY(cuda_check(cudaStreamSynchronize(s), "plan set-up"));

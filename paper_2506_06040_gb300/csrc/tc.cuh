@@ -116,6 +116,7 @@ struct TcArgs {
   float* fshade;           // frame: lighting pass output (FP32 RGBA per pixel) or NULL
   LightDev light;          // frame: lighting constants
   uint16_t* fout;          // frame: per-pixel output (nout FP16)
+  int fseg;                // frame: pixels per bulk copy of a whole uniform tile's output (0: pixel by pixel)
   int frame_w, tile_w, tile_h, tiles_x;
   int64_t frame_pixels;    // frame: pixel count (bounds of the checked build)
   int tmem_a;              // 1 = MMA A operands in TMEM (else shared memory)

@@ -202,6 +202,12 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
   // slot state that lives across chunks (mbarrier phases)
   uint32_t dph[kSlots] = {};
   bool first_chunk = true;
+  // batch: thread 0 takes a chunk's number while the chunk before it runs
+  int next_c = 0, nchunks = 0;
+  if (MODE == kModeBatch && tid == 0) {
+    nchunks = *p.nchunks_dev;
+    next_c = atomicAdd(p.chunk_counter, 1);
+  }
 
   for (;;) {
     // ---- take the next chunk (thread 0), load its material's MLP if it changed
@@ -222,11 +228,12 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           reload = 1;
         }
       } else {
-        const int c = atomicAdd(p.chunk_counter, 1);
-        if (c < *p.nchunks_dev) {
+        const int c = next_c;
+        if (c < nchunks) {
+          next_c = atomicAdd(p.chunk_counter, 1);
           const WorkChunk ch = p.chunks[c];
           reload = ch.mat != work.c.mat;
-          if (reload) work.m = p.mats[ch.mat];
+          if (reload) work.m.packed = p.mats[ch.mat].packed;
           work.c = ch;
           valid = 1;
         }
@@ -242,6 +249,11 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
     first_chunk = false;
     if (!work.valid) break;
     if (work.reload) {
+      if (MODE == kModeBatch) {  // the material's view, by all threads (published by the barrier below)
+        const uint32_t* from = reinterpret_cast<const uint32_t*>(p.mats + work.c.mat);
+        uint32_t* to = reinterpret_cast<uint32_t*>(&work.m);
+        for (int i = tid; i < (int)(sizeof(MatDev) / 4); i += W * kTile + 32 * W) to[i] = __ldg(from + i);
+      }
       // always waited (fixed budget), also after a timed-out D-ready wait: the
       // copy must land before the MMAs read the image and before the CTA exits
       if (!mbar_wait_bounded(wbar, wph, kDrainBudget)) failed = true;
@@ -477,16 +489,21 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           av[7] = 0u;
         }
       };
+      // frame chunks: this thread's pixel of each slot's tile and of the slot's next
+      // tile, whose list lookups are issued a tile ahead
+      int cur_px[kSlots] = {}, next_px[kSlots] = {};
+      const bool frame_chunk = MODE == kModeBatch && !grid_chunk;
+      auto pixel_of = [&](int64_t T) { return T < g_end ? (int)frame_pixel(p, work.c, T, gt) : -1; };
+
       // the packed A0 row of this thread's row of tile T: from the features of its
-      // texel, or (frame chunks, FP16 only) the row the feature pass left for its pixel
-      auto tile_row = [&](int64_t T, uint32_t (&av)[16]) {
+      // texel, or (frame chunks, FP16 only) the row the feature pass left for its pixel px
+      auto tile_row = [&](int64_t T, int px, uint32_t (&av)[16]) {
         if (MODE == kModeSingle || grid_chunk) {
           float f[12];
           tile_features(T, f);
           pack_a0(f, av);
         } else {
-          const int64_t px = frame_pixel(p, work.c, T, gt);
-          const uint2* r = p.ffeat + 3 * (px < 0 ? 0 : px);
+          const uint2* r = p.ffeat + 3 * (int64_t)max(px, 0);
 #pragma unroll
           for (int i = 0; i < 3; ++i) {
             const uint2 q = __ldg(r + i);
@@ -514,7 +531,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
         const uint32_t a0 = sbase + S.slots + q * S.slot + S.a0;
         if constexpr (TA || FORM == kF16) {
           uint32_t av[16];
-          tile_row(T, av);
+          tile_row(T, cur_px[s], av);
           if constexpr (TA) {
             store_a0(s, av);
             return;
@@ -778,18 +795,38 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
               if (k < nout) o[k] = hv[k];
           }
         } else {
-          const int64_t px = frame_pixel(p, work.c, T, gt);
-          if (px >= 0) {
-            uint16_t* o = p.fout + px * nout;
+          const int px = cur_px[s];
+          const bool whole = p.fseg && work.c.kind == kChunkUniform && __all_sync(0xffffffffu, px >= 0);
+          if (whole) {
+            // the warp's 32 pixels lie in 32 / fseg runs of a row, each contiguous
+            // in the output: staged and written with one bulk copy a run
+            const int runs = 32 / p.fseg;
+            if (lane < runs) bulk_wait_read0();
+            __syncwarp();
 #pragma unroll
             for (int k = 0; k < kMaxOut; ++k)
-              if (k < nout) o[k] = hv[k];
+              if (k < nout) sts16(stage_s + 2u * (uint32_t)(lane * nout + k), hv[k]);
+            fence_proxy_async_smem();
+            const int first = __shfl_sync(0xffffffffu, px, (lane * p.fseg) & 31);
+            if (lane < runs) {
+              const uint32_t bytes = 2u * (uint32_t)(p.fseg * nout);
+              bulk_s2g(p.fout + (int64_t)first * nout, stage_s + (uint32_t)lane * bytes, bytes);
+              bulk_commit();
+            }
+          }
+          if (px >= 0) {
+            uint16_t* o = p.fout + (int64_t)px * nout;
+            if (!whole) {
+#pragma unroll
+              for (int k = 0; k < kMaxOut; ++k)
+                if (k < nout) o[k] = hv[k];
+            }
             if (p.fshade) {  // lighting pass on the pixel's FP16 G-buffer channels
               float y[8];
 #pragma unroll
               for (int k = 0; k < 8; ++k) y[k] = __half2float(__ushort_as_half(hv[k]));
               const float3 c = shade_pixel(y, p.light);
-              *reinterpret_cast<float4*>(p.fshade + 4 * px) = make_float4(c.x, c.y, c.z, 1.f);
+              *reinterpret_cast<float4*>(p.fshade + 4 * (int64_t)px) = make_float4(c.x, c.y, c.z, 1.f);
             }
           }
         }
@@ -797,7 +834,13 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
 
 #pragma unroll
       for (int s = 0; s < kSlots; ++s)  // prime each of this warpgroup's own slots
-        if (g_begin + s < g_end) start_tile(s, g_begin + s);
+        if (g_begin + s < g_end) {
+          if (frame_chunk) {
+            cur_px[s] = pixel_of(g_begin + s);
+            next_px[s] = pixel_of(g_begin + s + kSlots);
+          }
+          start_tile(s, g_begin + s);
+        }
       for (int64_t base = g_begin; base < g_end; base += kSlots) {
         const bool two = base + 1 < g_end;
 #pragma unroll
@@ -825,11 +868,15 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
               if constexpr (TA) {
                 // the next tile's features while the output layer's MMAs run
                 // (stored into TMEM once those have read this tile's A)
-                if (l == NHID - 1 && base + s + kSlots < g_end) tile_row(base + s + kSlots, next_a0);
+                if (l == NHID - 1 && base + s + kSlots < g_end) tile_row(base + s + kSlots, next_px[s], next_a0);
               }
             } else {
               const bool more = base + s + kSlots < g_end;
               output_epilogue(s, base + s, TA && more);
+              if (frame_chunk) {
+                cur_px[s] = next_px[s];
+                next_px[s] = pixel_of(base + s + 2 * kSlots);
+              }
               if constexpr (!TA) {
                 if (more) start_tile(s, base + s + kSlots);
               }
