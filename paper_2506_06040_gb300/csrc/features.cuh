@@ -198,6 +198,7 @@ struct StripCache {
   uint32_t t1;     // own job: RGB8 of texel (jx, y1) -- the next pair's (jx, y0) when the key steps by one
   float c0[3];     // own job: texel (jx, y0), RGB / 255
   float dc[3];     // own job: texel (jx, y1) minus texel (jx, y0), RGB / 255
+  float hf, ys;    // own job (warp_strip_features): the level's height and shift - 1/2
 };
 
 __device__ __forceinline__ void strip_reset(StripCache& C) { C.i0 = -1; }
@@ -338,6 +339,8 @@ __device__ __forceinline__ void warp_strip_features(const DecodeArgs& a, int j, 
       if (lane >= total && lane < total + span) {
         job = k | (lane - total) << 2;
         jx = wrap_or_clamp(b0 + lane - total, L.w, a.wrap);
+        C.hf = (float)L.h;
+        C.ys = L.shift - 0.5f;
       }
       const float tx = texel_coord(u, L.w, L.shift);
       const float ftx = floorf(tx);
@@ -356,14 +359,14 @@ __device__ __forceinline__ void warp_strip_features(const DecodeArgs& a, int j, 
     return;
   }
   float cv0 = 0.f, cv1 = 0.f, cv2 = 0.f;
+  const float v = grid_coord((float)(j + a.row0), a.ch);
   if (C.job >= 0) {
-    const int k = C.job & 3;
-    const LevelView& L = a.lv[k];
-    const float ty = texel_coord(grid_coord((float)(j + a.row0), a.ch), L.h, L.shift);
+    const float ty = fmaf(v, C.hf, C.ys);
     const float fty = floorf(ty);
     const float fy = ty - fty;
     const int key = (int)fty;
     if (key != C.key) {
+      const LevelView& L = a.lv[C.job & 3];
       uint32_t t0;
       if (key == C.key + 1) {
         t0 = C.t1;
@@ -373,6 +376,9 @@ __device__ __forceinline__ void warp_strip_features(const DecodeArgs& a, int j, 
       }
       const int y1 = wrap_or_clamp(key + 1, L.h, a.wrap);
       const uint32_t t1 = bc1_texel(__ldg(L.blocks + block_index(L, C.jx >> 2, y1 >> 2)), C.jx & 3, y1 & 3);
+      // the next pair's lower texel: its block into L1 now, rows before it is read
+      const int y2 = wrap_or_clamp(key + 2, L.h, a.wrap);
+      if ((y2 ^ y1) >> 2) sm100::prefetch_l1(L.blocks + block_index(L, C.jx >> 2, y2 >> 2));
       C.key = key;
       C.t1 = t1;
 #pragma unroll
@@ -385,12 +391,6 @@ __device__ __forceinline__ void warp_strip_features(const DecodeArgs& a, int j, 
     cv0 = fmaf(fy, C.dc[0], C.c0[0]);
     cv1 = fmaf(fy, C.dc[1], C.c0[1]);
     cv2 = fmaf(fy, C.dc[2], C.c0[2]);
-    const float tyn = texel_coord(grid_coord((float)(j + a.row0 + 1), a.ch), L.h, L.shift);
-    const int keyn = (int)floorf(tyn);
-    if (keyn != key && j + 1 < a.grid_h) {
-      const int y1 = wrap_or_clamp(keyn + 1, L.h, a.wrap);
-      sm100::prefetch_l1(L.blocks + block_index(L, C.jx >> 2, y1 >> 2));
-    }
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {

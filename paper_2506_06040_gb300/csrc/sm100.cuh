@@ -289,7 +289,7 @@ __device__ __forceinline__ void split_relu_f16x2(float a, float b, uint32_t& hi,
       : "=f"(ra), "=f"(rb)
       : "r"(hi), "h"((unsigned short)0xBC00u), "f"(a), "f"(b));
   const uint32_t r = cvt_f16x2(ra, rb);
-  asm("max.f16x2 %0, %1, %2;" : "=r"(lo) : "r"(r), "r"(hi ^ 0x80008000u));
+  asm("{\n .reg .b32 n;\n neg.f16x2 n, %2;\n max.f16x2 %0, %1, n;\n}" : "=r"(lo) : "r"(r), "r"(hi));
 }
 //  E4M3 (of an FP16 pair v16): hi = E4M3(v16), lo = E4M3(v16 - hi); the
 //  residual of rounding an FP16 value to E4M3 is itself an FP16 value, so the

@@ -151,7 +151,9 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
   const TcSmem S = tc_smem(L, W, NSL, TA);
   const uint32_t sbase = smem_u32(smem);
   const int tid = threadIdx.x;
-  const int warp = tid / 32, lane = tid % 32;
+  // warp-uniform, and known to be: the MMA warps' descriptors and the addresses
+  // derived from it stay in uniform registers
+  const int warp = __shfl_sync(0xffffffffu, tid / 32, 0), lane = tid % 32;
   const uint32_t dbar0 = sbase + S.bars, wbar = dbar0 + NS * 8;
   // named barriers: 0 = __syncthreads, 1 + W + q = A-ready of slot q; with TA
   // (one slot per warpgroup) 1 + q = D-ready of slot q
@@ -733,24 +735,40 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
         }
         const float alp = alpha[NHID];
         const float* b = bias + NHID * kHid;
-        uint16_t hv[kMaxOut];
+        uint32_t hp[kMaxOut / 2];  // FP16 channel pairs
         if constexpr (FP8) {
 #pragma unroll
           for (int k = 0; k < kMaxOut; k += 2) {
             const float2 v = __ffma2_rn(make_float2(__uint_as_float(r[k]), __uint_as_float(r[k + 1])),
                                         make_float2(alp, alp), *reinterpret_cast<const float2*>(b + k));
-            hv[k] = __half_as_ushort(__float2half_rn(v.x));
-            hv[k + 1] = __half_as_ushort(__float2half_rn(v.y));
+            hp[k / 2] = cvt_f16x2(v.x, v.y);
           }
         } else {
 #pragma unroll
-          for (int k = 0; k < kMaxOut; ++k) hv[k] = __half_as_ushort(__float2half_rn(__uint_as_float(r[k])));
+          for (int k = 0; k < kMaxOut; k += 2)
+            hp[k / 2] = cvt_f16x2(__uint_as_float(r[k]), __uint_as_float(r[k + 1]));
         }
+        auto channel = [&](int k) { return (uint16_t)(k & 1 ? hp[k / 2] >> 16 : hp[k / 2] & 0xFFFFu); };
+        // this lane's nout halves into the warp's stage, as 32-bit words wherever
+        // they are aligned: with an odd count the odd lanes' rows start between two
+        // words, so their first half goes alone and the words shift by one half
+        auto stage_row = [&]() {
+          const bool odd = (lane & nout & 1) != 0;
+          const uint32_t row = stage_s + 2u * (uint32_t)(lane * nout), at = row + (odd ? 2u : 0u);
+          const uint32_t sel = odd ? 0x5432u : 0x3210u;
+          uint32_t single = hp[0];
+#pragma unroll
+          for (int i = 0; i < kMaxOut / 2; ++i) {
+            if (2 * i + 1 < nout) sts32(at + 4u * i, __byte_perm(hp[i], i + 1 < kMaxOut / 2 ? hp[i + 1] : 0u, sel));
+            if (2 * i + 1 == nout && !odd) single = hp[i];
+          }
+          if (nout & 1) sts16(odd ? row : row + 2u * (uint32_t)(nout - 1), (uint16_t)single);
+        };
         if constexpr (OUT32) {
           // FP32 output (single-material grids and uv lists): the accumulator as is
           const int64_t t0 = tile_first_texel(D, hdiv, footprint, work.c.first + T);
           const int64_t tex = t0 + gt;
-          if (t0 + kTile <= D.n) {
+          if (footprint || t0 + kTile <= D.n) {  // (footprint tiles are whole)
             // the warp's 32 texels x nout floats are contiguous: one bulk copy of
             // 128 nout bytes at a 128-byte multiple of the 16-byte aligned output
             if (lane == 0) bulk_wait_read0();
@@ -773,15 +791,13 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
         } else if (MODE == kModeSingle || grid_chunk) {
           const int64_t t0 = tile_first_texel(D, hdiv, footprint, work.c.first + T);
           const int64_t tex = t0 + gt;
-          if (t0 + kTile <= D.n) {
+          if (footprint || t0 + kTile <= D.n) {  // (footprint tiles are whole)
             // the warp's 32 texels x nout halves are contiguous in the output:
             // stage them and write them with one bulk copy (64 nout bytes at a
             // 64-byte multiple of the 16-byte aligned output)
             if (lane == 0) bulk_wait_read0();  // the warp's previous bulk copy has read the stage
             __syncwarp();
-#pragma unroll
-            for (int k = 0; k < kMaxOut; ++k)
-              if (k < nout) sts16(stage_s + 2u * (uint32_t)(lane * nout + k), hv[k]);
+            stage_row();
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
@@ -792,7 +808,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             uint16_t* o = reinterpret_cast<uint16_t*>(D.out) + tex * nout;
 #pragma unroll
             for (int k = 0; k < kMaxOut; ++k)
-              if (k < nout) o[k] = hv[k];
+              if (k < nout) o[k] = channel(k);
           }
         } else {
           const int px = cur_px[s];
@@ -803,9 +819,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             const int runs = 32 / p.fseg;
             if (lane < runs) bulk_wait_read0();
             __syncwarp();
-#pragma unroll
-            for (int k = 0; k < kMaxOut; ++k)
-              if (k < nout) sts16(stage_s + 2u * (uint32_t)(lane * nout + k), hv[k]);
+            stage_row();
             fence_proxy_async_smem();
             const int first = __shfl_sync(0xffffffffu, px, (lane * p.fseg) & 31);
             if (lane < runs) {
@@ -819,12 +833,12 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             if (!whole) {
 #pragma unroll
               for (int k = 0; k < kMaxOut; ++k)
-                if (k < nout) o[k] = hv[k];
+                if (k < nout) o[k] = channel(k);
             }
             if (p.fshade) {  // lighting pass on the pixel's FP16 G-buffer channels
               float y[8];
 #pragma unroll
-              for (int k = 0; k < 8; ++k) y[k] = __half2float(__ushort_as_half(hv[k]));
+              for (int k = 0; k < 8; ++k) y[k] = __half2float(__ushort_as_half(channel(k)));
               const float3 c = shade_pixel(y, p.light);
               *reinterpret_cast<float4*>(p.fshade + 4 * (int64_t)px) = make_float4(c.x, c.y, c.z, 1.f);
             }
@@ -861,7 +875,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
               }
               dph[s] ^= 1u;
             }
-            failed = __any_sync(0xffffffffu, failed);  // one failure state per warp
+            if constexpr (!TA) failed = __any_sync(0xffffffffu, failed);  // one failure state per warp
             tc_fence_after();
             if (l < NHID) {
               hidden_epilogue(s, l);
