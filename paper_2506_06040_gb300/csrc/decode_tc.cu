@@ -277,6 +277,20 @@ static void tc_shape_of(const nbtc_context* ctx, int form, int& W, int& slots) {
   }
 }
 
+// Whether a decode walks its grid in column strips of 128-texel tiles, whose
+// latent columns are decoded once per pair of rows.  The last strip of a row that
+// 128 does not divide is decoded past the row's end, so the rule bounds what that
+// wastes: 2.1 M texels in whole strips take 61 us in FP16 (12-64-64-9) and 122 us in
+// split FP16 (12-64-64-64-9), sampled texel by texel (16 BC1 taps each) 188 us and
+// 272 us, so strips win up to 2.2 decoded texels per texel in the slower form and
+// the line is at 2.  It does not depend on the rows, so a band of rows is decoded
+// as the whole grid is.
+static bool strip_grid(const DecodeArgs& a) {
+  if (a.uv || a.grid_w < 1) return false;
+  const int64_t padded = (int64_t)((a.grid_w + kTile - 1) / kTile) * kTile;
+  return padded <= 2 * (int64_t)a.grid_w;
+}
+
 nbtc_status launch_decode_tc(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, int precision,
                              const void* packed, cudaStream_t s) {
   int nhid;
@@ -290,11 +304,13 @@ nbtc_status launch_decode_tc(nbtc_context* ctx, const DecodeArgs& a, const nbtc_
   p.d = a;
   p.packed = packed;
   p.nout = mlp->dims[nhid + 1];
-  p.tiles = (a.n + kTile - 1) / kTile;
   p.budget = ctx->wait_budget > 0 ? ctx->wait_budget : ctx->wait_budget < 0 ? 0 : kDefaultWaitBudget;
-  bool fp = a.uv == nullptr && (a.grid_w % kTile) == 0;
+  bool fp = strip_grid(a);
   for (int k = 0; k < 4; ++k) fp = fp && a.lv[k].w <= a.grid_w;
   p.footprint = fp ? 1 : 0;
+  p.tiles = fp ? (int64_t)((a.grid_w + kTile - 1) / kTile) * a.grid_h : (a.n + kTile - 1) / kTile;
+  // (the output is 16-byte aligned; 32 rows of FP16 are 64 nout bytes)
+  p.whole_rows = fp ? a.grid_w % kTile == 0 : a.n % kTile == 0;
   p.hdiv = make_fastdiv(fp && a.grid_h > 0 ? (uint32_t)a.grid_h : 1u);
   p.mode = kModeSingle;
   if (p.tiles >= (int64_t)1 << 31) return fail(NBTC_ERR_UNSUPPORTED, "more than 2^31 tiles");

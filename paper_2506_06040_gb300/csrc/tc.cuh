@@ -20,8 +20,9 @@ constexpr int kMaxOut = 16;
 // FP32 (no output rounding): the FP32-accurate form.
 enum TcForm { kF16 = 0, kF8 = 1, kF16Split = 2, kF8Split = 3, kF32Split = 4 };
 
-// Bytes of per-warp output staging: 32 texels x up to 16 channels of FP16, or FP32.
-__host__ __device__ constexpr int stage_bytes(int form) { return form == kF32Split ? 2048 : 1024; }
+// Bytes of per-warp output staging: 32 texels x up to 16 channels of FP16, or FP32,
+// shifted by up to 15 bytes to match the destination.
+__host__ __device__ constexpr int stage_bytes(int form) { return (form == kF32Split ? 2048 : 1024) + 16; }
 
 // Byte layout of a packed MLP (identical in global memory and shared memory).
 // FP16 forms: every layer's bias enters the MMA as FP16 operand(s) -- layer 1
@@ -99,6 +100,7 @@ struct TcArgs {
   const void* packed;
   int nout;
   int footprint;       // 1: row-footprint feature stage
+  int whole_rows;      // single material: every warp's 32 output rows exist and start on 16 bytes
   FastDiv hdiv;        // footprint mode: division by grid_h (tile number -> column block)
   int64_t tiles;
   int64_t per_cta;     // tiles per CTA (contiguous range)

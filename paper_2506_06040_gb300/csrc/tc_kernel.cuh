@@ -34,13 +34,50 @@ using namespace sm100;
 // row-footprint mode consecutive numbers run down a column of 128-texel tiles
 // (number -> row = T % H, column block = T / H), so the consecutive tiles a
 // warpgroup decodes are consecutive rows of one column strip (the feature
-// stage's column cache relies on this).  Returns the first output texel of tile T.
-__device__ __forceinline__ int64_t tile_first_texel(const DecodeArgs& d, const FastDiv& hdiv, bool footprint,
-                                                    int64_t T) {
-  if (!footprint) return T * 128;
-  const uint32_t t = (uint32_t)T;
-  const uint32_t col = fastdiv(t, hdiv), row = t - col * (uint32_t)d.grid_h;
-  return (int64_t)row * d.grid_w + (int64_t)col * 128;
+// stage's column cache relies on this).  The last column of tiles may reach
+// past the row's end: its texels there are decoded and not stored.  WarpRows:
+// the first output texel of a warp's 32 rows of tile T and how many of them exist.
+struct WarpRows {
+  int64_t first;
+  int live;  // <= 32; <= 0: none
+};
+__device__ __forceinline__ WarpRows warp_rows(const DecodeArgs& d, const FastDiv& hdiv, bool footprint, int64_t T,
+                                              int wq) {
+  WarpRows r;
+  if (footprint) {
+    const uint32_t t = (uint32_t)T;
+    const uint32_t col = fastdiv(t, hdiv), row = t - col * (uint32_t)d.grid_h;
+    const int x = (int)col * 128 + 32 * wq;
+    r.first = (int64_t)row * d.grid_w + x;
+    r.live = min(d.grid_w - x, 32);
+  } else {
+    r.first = T * 128 + 32 * wq;
+    r.live = (int)min(d.n - r.first, (int64_t)32);
+  }
+  return r;
+}
+
+// `bytes` staged bytes (from stage + off, off = dst % 16, a multiple of UNIT) to
+// global memory: the whole 16-byte pieces by one bulk copy of lane 0, what is
+// left before and after them (rows that do not start on 16 bytes) UNIT bytes a
+// lane.  All lanes have staged, fenced and synchronised.
+template <int UNIT>
+__device__ __forceinline__ void put_staged(unsigned char* dst, uint32_t stage, uint32_t off, uint32_t bytes, int lane) {
+  const uint32_t end = off + bytes, b16 = (off + 15u) & ~15u, e16 = end & ~15u;
+  unsigned char* g0 = dst - off;  // global address of stage + 0
+  if (lane == 0 && e16 > b16) {
+    bulk_s2g(g0 + b16, stage + b16, e16 - b16);
+    bulk_commit();
+  }
+  if ((off | end) & 15u) {
+    constexpr uint32_t N = 16 / UNIT;
+    const bool head = (uint32_t)lane < N;
+    const uint32_t at = head ? off + UNIT * (uint32_t)lane : max(e16, b16) + UNIT * ((uint32_t)lane - N);
+    if ((uint32_t)lane < 2 * N && at < (head ? min(b16, end) : end)) {
+      if constexpr (UNIT == 2) *reinterpret_cast<uint16_t*>(g0 + at) = lds16(stage + at);
+      else *reinterpret_cast<uint32_t*>(g0 + at) = lds32(stage + at);
+    }
+  }
 }
 
 // Frame pixel decoded by row `gt` of tile `T` of chunk `c` (-1: none).  A
@@ -439,6 +476,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
       const DecodeArgs& D = MODE == kModeSingle ? p.d : work.m.d;
       const FastDiv& hdiv = MODE == kModeSingle ? p.hdiv : work.m.hdiv;
       const int nout = work.m.nout;
+      const bool whole_rows = p.whole_rows != 0;
       const int64_t g_begin = min((int64_t)wg * per_wg, range_end);
       const int64_t g_end = min(g_begin + per_wg, range_end);
       StripCache cache;
@@ -752,7 +790,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
         // this lane's nout halves into the warp's stage, as 32-bit words wherever
         // they are aligned: with an odd count the odd lanes' rows start between two
         // words, so their first half goes alone and the words shift by one half
-        auto stage_row = [&]() {
+        auto stage_row0 = [&]() {
           const bool odd = (lane & nout & 1) != 0;
           const uint32_t row = stage_s + 2u * (uint32_t)(lane * nout), at = row + (odd ? 2u : 0u);
           const uint32_t sel = odd ? 0x5432u : 0x3210u;
@@ -764,13 +802,32 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           }
           if (nout & 1) sts16(odd ? row : row + 2u * (uint32_t)(nout - 1), (uint16_t)single);
         };
+        // the same from byte `off` of the stage (rows whose output does not start on
+        // 16 bytes): this lane's nout halves, as 32-bit
+        // words wherever they are aligned: a row that starts between two words
+        // (every other one with an odd count) puts its first half alone and shifts
+        // its words by one half
+        auto stage_row = [&](uint32_t off) {
+          const uint32_t row = stage_s + off + 2u * (uint32_t)(lane * nout);
+          const bool odd = (row & 2u) != 0u, even_n = (nout & 1) == 0;
+          const uint32_t at = row + (odd ? 2u : 0u), sel = odd ? 0x5432u : 0x3210u;
+          const int lim = nout - (even_n && odd ? 1 : 0);
+          uint32_t single = hp[0], last = 0u;
+#pragma unroll
+          for (int i = 0; i < kMaxOut / 2; ++i) {
+            if (2 * i + 1 < lim) sts32(at + 4u * i, __byte_perm(hp[i], i + 1 < kMaxOut / 2 ? hp[i + 1] : 0u, sel));
+            if (2 * i + 1 == nout && !odd) single = hp[i];
+            if (2 * i + 2 == nout) last = hp[i] >> 16;
+          }
+          if (odd || !even_n) sts16(odd ? row : row + 2u * (uint32_t)(nout - 1), (uint16_t)single);
+          if (odd && even_n) sts16(row + 2u * (uint32_t)(nout - 1), (uint16_t)last);
+        };
         if constexpr (OUT32) {
-          // FP32 output (single-material grids and uv lists): the accumulator as is
-          const int64_t t0 = tile_first_texel(D, hdiv, footprint, work.c.first + T);
-          const int64_t tex = t0 + gt;
-          if (footprint || t0 + kTile <= D.n) {  // (footprint tiles are whole)
-            // the warp's 32 texels x nout floats are contiguous: one bulk copy of
-            // 128 nout bytes at a 128-byte multiple of the 16-byte aligned output
+          // FP32 output (single-material grids and uv lists): the accumulator as is.
+          // The warp's live texels x nout floats are contiguous in the output:
+          // staged and written together
+          const WarpRows wr = warp_rows(D, hdiv, footprint, work.c.first + T, wq);
+          if (whole_rows) {  // 128 nout bytes at a multiple of 16: one bulk copy
             if (lane == 0) bulk_wait_read0();
             __syncwarp();
 #pragma unroll
@@ -779,36 +836,42 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
-              bulk_s2g(reinterpret_cast<float*>(D.out) + (t0 + 32 * wq) * nout, stage_s, 128u * (uint32_t)nout);
+              bulk_s2g(reinterpret_cast<float*>(D.out) + wr.first * nout, stage_s, 128u * (uint32_t)nout);
               bulk_commit();
             }
-          } else if (tex < D.n) {
-            float* o = reinterpret_cast<float*>(D.out) + tex * nout;
-#pragma unroll
-            for (int k = 0; k < kMaxOut; ++k)
-              if (k < nout) o[k] = __uint_as_float(r[k]);
-          }
-        } else if (MODE == kModeSingle || grid_chunk) {
-          const int64_t t0 = tile_first_texel(D, hdiv, footprint, work.c.first + T);
-          const int64_t tex = t0 + gt;
-          if (footprint || t0 + kTile <= D.n) {  // (footprint tiles are whole)
-            // the warp's 32 texels x nout halves are contiguous in the output:
-            // stage them and write them with one bulk copy (64 nout bytes at a
-            // 64-byte multiple of the 16-byte aligned output)
+          } else if (wr.live > 0) {
+            unsigned char* dst = reinterpret_cast<unsigned char*>(D.out) + 4 * (wr.first * nout);
+            const uint32_t off = (uint32_t)(reinterpret_cast<uintptr_t>(dst) & 15u);
             if (lane == 0) bulk_wait_read0();  // the warp's previous bulk copy has read the stage
             __syncwarp();
-            stage_row();
+#pragma unroll
+            for (int k = 0; k < kMaxOut; ++k)
+              if (k < nout) sts32(stage_s + off + 4u * (uint32_t)(lane * nout + k), r[k]);
+            fence_proxy_async_smem();
+            __syncwarp();
+            put_staged<4>(dst, stage_s, off, 4u * (uint32_t)(wr.live * nout), lane);
+          }
+        } else if (MODE == kModeSingle || grid_chunk) {
+          const WarpRows wr = warp_rows(D, hdiv, footprint, work.c.first + T, wq);
+          if (MODE == kModeBatch || whole_rows) {  // 64 nout bytes at a multiple of 16: one bulk copy
+            if (lane == 0) bulk_wait_read0();
+            __syncwarp();
+            stage_row0();
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
-              bulk_s2g(reinterpret_cast<uint16_t*>(D.out) + (t0 + 32 * wq) * nout, stage_s, 64u * (uint32_t)nout);
+              bulk_s2g(reinterpret_cast<uint16_t*>(D.out) + wr.first * nout, stage_s, 64u * (uint32_t)nout);
               bulk_commit();
             }
-          } else if (tex < D.n) {
-            uint16_t* o = reinterpret_cast<uint16_t*>(D.out) + tex * nout;
-#pragma unroll
-            for (int k = 0; k < kMaxOut; ++k)
-              if (k < nout) o[k] = channel(k);
+          } else if (wr.live > 0) {
+            unsigned char* dst = reinterpret_cast<unsigned char*>(D.out) + 2 * (wr.first * nout);
+            const uint32_t off = (uint32_t)(reinterpret_cast<uintptr_t>(dst) & 15u);
+            if (lane == 0) bulk_wait_read0();
+            __syncwarp();
+            stage_row(off);
+            fence_proxy_async_smem();
+            __syncwarp();
+            put_staged<2>(dst, stage_s, off, 2u * (uint32_t)(wr.live * nout), lane);
           }
         } else {
           const int px = cur_px[s];
@@ -819,7 +882,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             const int runs = 32 / p.fseg;
             if (lane < runs) bulk_wait_read0();
             __syncwarp();
-            stage_row();
+            stage_row0();
             fence_proxy_async_smem();
             const int first = __shfl_sync(0xffffffffu, px, (lane * p.fseg) & 31);
             if (lane < runs) {

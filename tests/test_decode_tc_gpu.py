@@ -92,6 +92,52 @@ def test_fp16_ragged(nb, ctx, gw, gh):
     _check_fp16(got, wl.material, _grid_x(wl.material, gw, gh))
 
 
+@pytest.mark.parametrize("gw,gh,nout", [(65, 40, 9), (63, 9, 9), (130, 33, 9), (150, 40, 9), (161, 33, 8), (300, 9, 3), (385, 5, 16), (1500, 3, 9),
+                                        (146, 21, 9), (75, 30, 9), (31, 3, 9)])
+@pytest.mark.parametrize("form", ["FP16", "FP32_TC"])
+def test_ragged_strips(nb, ctx, gw, gh, nout, form):
+    """Widths that 128 does not divide, on both sides of the strip rule: rows that
+    start between 16-byte pieces (any 2-byte phase in FP16, 4-byte in FP32), last
+    columns of one to 127 texels, whole warps past the row's end; nothing is
+    written before or after the output."""
+    wl = synth.small_decode_workload(256, [12, 64, nout], seed=350 + gw, level_sides=[64, 32, 16, 8])
+    mat = nb.Material.from_synth(wl.material)
+    code = getattr(nb, form)
+    packed = nb.pack_mlp(ctx, mat, code)
+    dt = torch.float16 if form == "FP16" else torch.float32
+    buf = torch.full((gw * gh * nout + 64,), 7.0, device="cuda", dtype=dt)
+    out = buf[32:32 + gw * gh * nout].view(gw * gh, nout)
+    nb.decode(ctx, mat, code, packed, grid=(gw, gh), out=out)
+    band = nb.decode(ctx, mat, code, packed, grid=(gw, gh), rows=(gh // 2, gh - gh // 2))
+    ctx.sync()
+    assert bool((buf[:32] == 7).all()) and bool((buf[-32:] == 7).all())
+    assert torch.equal(band, out[(gh // 2) * gw:])
+    got, x = out.float().cpu().numpy(), _grid_x(wl.material, gw, gh)
+    if form == "FP16":
+        _check(got, wl.material, x, "fp16")
+    else:
+        ref = oracle.mlp.forward(x, wl.material.mlp.weights, wl.material.mlp.biases)
+        assert np.abs(got.astype(np.float64) - ref).max() <= 1e-5
+
+
+@pytest.mark.parametrize("nout", [1, 2, 3, 8, 15, 16])
+@pytest.mark.parametrize("form,name", [("FP16", "fp16"), ("FP16_SPLIT", "fp16s")])
+def test_output_channel_counts(nb, ctx, nout, form, name):
+    """Odd and even channel counts up to 16: odd ones put every other row of the
+    output stage between two 32-bit words.  Whole tiles and a ragged uv list."""
+    wl = synth.small_decode_workload(256, [12, 64, nout], seed=340 + nout)
+    mat = nb.Material.from_synth(wl.material)
+    code = getattr(nb, form)
+    packed = nb.pack_mlp(ctx, mat, code)
+    uv = synth.random_uv(341, 517)
+    y = nb.decode(ctx, mat, code, packed, grid=(256, 9))
+    z = nb.decode(ctx, mat, code, packed, uv=torch.from_numpy(uv).cuda())
+    ctx.sync()
+    _check(y.float().cpu().numpy(), wl.material, _grid_x(wl.material, 256, 9), name)
+    _check(z.float().cpu().numpy(), wl.material,
+           oracle.decode.features_at(wl.material, uv[:, 0].astype(np.float64), uv[:, 1].astype(np.float64)), name)
+
+
 @pytest.mark.parametrize("address", ["clamp", "wrap"])
 def test_fp16_uv_list(nb, ctx, address):
     wl = synth.small_decode_workload(256, [12, 64, 64, 64, 9], seed=320, address=address)
