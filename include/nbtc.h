@@ -62,9 +62,12 @@ typedef enum {
  * rounding loses (max abs error vs FP64 on a He-initialised 12-64-64-64-9
  * decode: FP16 3.2e-3 -> 9.8e-4, the FP16 output rounding; E4M3 0.37 -> 1.2e-2;
  * before the output rounding the FP16 split is within ~1e-6, which NBTC_FP32_TC
- * keeps by writing FP32). */
+ * keeps by writing FP32, with every neuron scaled into FP16's range by a power of
+ * two). */
 typedef enum {
-  NBTC_FP32 = 0,            /* FP32 SIMT arithmetic (FFMA), FP32 output              */
+  NBTC_FP32 = 0,            /* FP32 weights in, FP32 accuracy, FP32 output: FP32 FMAs
+                               (FFMA); at hidden width 64, where it is at least as
+                               accurate, NBTC_FP32_TC's arithmetic                    */
   NBTC_FP16 = 1,            /* FP16 operands on tcgen05, FP32 accumulate, FP16 output */
   NBTC_FP8_E4M3 = 2,        /* E4M3 operands on tcgen05 with per-layer power-of-two
                                scales, FP32 accumulate, FP16 output                   */
@@ -126,9 +129,7 @@ typedef struct nbtc_context nbtc_context;
  * MMA A operands of the tensor-core forms (FP16, FP8_E4M3, both split forms, FP32_TC) in
  * shared memory instead of tensor memory; NBTC_TC_GROUPS=3 runs the
  * shared-memory-operand FP16 / FP8 decodes with 3 warpgroups per CTA instead of
- * 4; NBTC_FP32_GROUPS=1 runs the FP32 wide decode as one 512-thread group per
- * CTA instead of two independent 256-thread groups; NBTC_TRAIN_SIMT=1 runs
- * every training step on the FP32 SIMT kernel (default: the tensor-core kernel
+ * 4; NBTC_TRAIN_SIMT=1 runs every training step on the FP32 SIMT kernel (default: the tensor-core kernel
  * whenever the workspace holds the gathered samples; results agree to FP32
  * rounding, not bit for bit). */
 nbtc_status nbtc_create(int device, nbtc_context** ctx);

@@ -160,7 +160,6 @@ nbtc_status nbtc_create(int device, nbtc_context** out) {
   ctx->sm_count = prop.multiProcessorCount;
   if (const char* e = getenv("NBTC_TC_GROUPS")) ctx->tc_groups = atoi(e) == 3 ? 3 : 4;
   if (const char* e = getenv("NBTC_TC_TMEM_A")) ctx->tc_tmem_a = atoi(e) == 0 ? 0 : 1;
-  if (const char* e = getenv("NBTC_FP32_GROUPS")) ctx->fp32_groups = atoi(e) == 1 ? 1 : 2;
   if (const char* e = getenv("NBTC_TRAIN_SIMT")) ctx->train_tc = atoi(e) == 1 ? 0 : 1;
   if ((st = cuda_check(cudaMalloc(&ctx->status_dev, sizeof(int)), "cudaMalloc(status)"))) {
     delete ctx;
@@ -306,7 +305,8 @@ nbtc_status nbtc_fp8_calibrate(nbtc_context* ctx, const nbtc_latents* lat, const
 // Where a decode may write: device (or managed) memory, or -- FP32 decodes,
 // whose kernels store with plain global stores -- pinned host memory, which the
 // kernel writes directly over the host link (its device address replaces out).
-static nbtc_status resolve_out(int32_t precision, DecodeArgs& a) {
+static nbtc_status resolve_out(int32_t precision, DecodeArgs& a, bool& host_out) {
+  host_out = false;
   cudaPointerAttributes pa;
   const cudaError_t e = cudaPointerGetAttributes(&pa, a.out);
   if (e != cudaSuccess) {
@@ -324,6 +324,7 @@ static nbtc_status resolve_out(int32_t precision, DecodeArgs& a) {
       return fail(NBTC_ERR_UNSUPPORTED,
                   "pinned host output is for the FP32 SIMT decode; tensor-core forms decode into device memory");
     a.out = pa.devicePointer;
+    host_out = true;
     if (!aligned(a.out, 16)) return fail(NBTC_ERR_INVALID_ARG, "out not 16-byte aligned");
     return NBTC_OK;
   }
@@ -339,10 +340,11 @@ nbtc_status nbtc_decode(nbtc_context* ctx, const nbtc_latents* lat, const nbtc_m
   DecodeArgs a;
   if ((st = make_decode_args(ctx, lat, mlp, uv_dev, n, grid_w, grid_h, out_dev, a))) return st;
   if (n == 0) return NBTC_OK;
-  if ((st = resolve_out(precision, a))) return st;
+  bool host_out;
+  if ((st = resolve_out(precision, a, host_out))) return st;
   switch (precision) {
     case NBTC_FP32:
-      return launch_decode_fp32(ctx, a, mlp, (cudaStream_t)stream);
+      return launch_decode_fp32(ctx, a, mlp, host_out, (cudaStream_t)stream);
     case NBTC_FP16:
     case NBTC_FP8_E4M3:
     case NBTC_FP16_SPLIT:
@@ -366,12 +368,13 @@ nbtc_status nbtc_decode_rows(nbtc_context* ctx, const nbtc_latents* lat, const n
   DecodeArgs a;
   if ((st = make_decode_args(ctx, lat, mlp, nullptr, (int64_t)grid_w * rows, grid_w, rows, out_dev, a))) return st;
   if (rows == 0) return NBTC_OK;
-  if ((st = resolve_out(precision, a))) return st;
+  bool host_out;
+  if ((st = resolve_out(precision, a, host_out))) return st;
   a.row0 = row0;
   a.ch = make_grid_coord(grid_h);
   switch (precision) {
     case NBTC_FP32:
-      return launch_decode_fp32(ctx, a, mlp, (cudaStream_t)stream);
+      return launch_decode_fp32(ctx, a, mlp, host_out, (cudaStream_t)stream);
     case NBTC_FP16:
     case NBTC_FP8_E4M3:
     case NBTC_FP16_SPLIT:

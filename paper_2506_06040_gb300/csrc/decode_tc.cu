@@ -2,6 +2,7 @@
 // of shared memory), launch dispatch.  The kernel is in tc_kernel.cuh.
 #include <cstring>
 
+#include "f32s_pack.cuh"
 #include "host.h"
 #include "sm100.cuh"
 #include "tc.cuh"
@@ -74,6 +75,16 @@ __global__ void k_pack_mlp(const float* __restrict__ W, const float* __restrict_
   // clear the image
   for (int e = threadIdx.x; e < L.bytes(); e += blockDim.x) out[e] = 0;
   __syncthreads();
+  if (form == kF32Split) {
+    __shared__ F32sScratch S;
+    f32s_scales(W, B, nhid, hid, nout, threadIdx.x, blockDim.x, S);
+    if (S.bad) {  // weights that are not finite (or beyond any FP16 scale): unscaled, as the values fall
+      for (int e = threadIdx.x; e < 5 * kHid; e += blockDim.x) S.a[e / kHid][e % kHid] = 0;
+      __syncthreads();
+    }
+    f32s_pack(out, L, W, B, hid, nout, threadIdx.x, blockDim.x, S);
+    return;
+  }
   const int R1 = L.w1_row();
   off = 0;
   for (int l = 0; l < nl; ++l) {
@@ -277,6 +288,9 @@ static void tc_shape_of(const nbtc_context* ctx, int form, int& W, int& slots) {
   }
 }
 
+static nbtc_status launch_decode_form(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, int nhid, int form,
+                                      const void* packed, bool host_out, cudaStream_t s);
+
 // Whether a decode walks its grid in column strips of 128-texel tiles, whose
 // latent columns are decoded once per pair of rows.  The last strip of a row that
 // 128 does not divide is decoded past the row's end, so the rule bounds what that
@@ -291,6 +305,19 @@ static bool strip_grid(const DecodeArgs& a) {
   return padded <= 2 * (int64_t)a.grid_w;
 }
 
+// NBTC_FP32 (packed and host_out as nbtc_decode takes them): the FP32-accurate
+// form with the MLP laid out by each CTA; UNSUPPORTED, with nothing launched, for
+// shapes that stay with the FFMA kernels.  Taken at hidden width 64, where it is
+// as accurate as they are (f32s_pack.cuh) and 4096^2 12-64-64-9 takes 650 us
+// against 4060; narrower networks are less accurate here than in FFMA.  The rule is
+// the shape alone, so bands, host outputs and uv lists give the whole grid's bits.
+nbtc_status launch_decode_fp32_tc(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, bool host_out,
+                                  cudaStream_t s) {
+  int nhid;
+  if (tc_shape(mlp, nhid) || mlp->dims[1] != kHid) return NBTC_ERR_UNSUPPORTED;
+  return launch_decode_form(ctx, a, mlp, nhid, kF32Split, nullptr, host_out, s);
+}
+
 nbtc_status launch_decode_tc(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, int precision,
                              const void* packed, cudaStream_t s) {
   int nhid;
@@ -299,10 +326,22 @@ nbtc_status launch_decode_tc(nbtc_context* ctx, const DecodeArgs& a, const nbtc_
   const int form = tc_form(precision);
   if (form < 0) return fail(NBTC_ERR_INVALID_ARG, "not a tensor-core precision");
   if (!packed || !aligned(packed, 16)) return fail(NBTC_ERR_INVALID_ARG, "packed MLP NULL or not 16-byte aligned");
+  return launch_decode_form(ctx, a, mlp, nhid, form, packed, false, s);
+}
+
+static nbtc_status launch_decode_form(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, int nhid, int form,
+                                      const void* packed, bool host_out, cudaStream_t s) {
   TcArgs p;
   memset(&p, 0, sizeof(p));
   p.d = a;
   p.packed = packed;
+  p.mode = packed ? kModeSingle : kModeInPlace;
+  if (!packed) {
+    p.W = mlp->weights;
+    p.B = mlp->biases;
+    p.hid = mlp->dims[1];
+    p.host_out = host_out ? 1 : 0;
+  }
   p.nout = mlp->dims[nhid + 1];
   p.budget = ctx->wait_budget > 0 ? ctx->wait_budget : ctx->wait_budget < 0 ? 0 : kDefaultWaitBudget;
   bool fp = strip_grid(a);
@@ -312,11 +351,10 @@ nbtc_status launch_decode_tc(nbtc_context* ctx, const DecodeArgs& a, const nbtc_
   // (the output is 16-byte aligned; 32 rows of FP16 are 64 nout bytes)
   p.whole_rows = fp ? a.grid_w % kTile == 0 : a.n % kTile == 0;
   p.hdiv = make_fastdiv(fp && a.grid_h > 0 ? (uint32_t)a.grid_h : 1u);
-  p.mode = kModeSingle;
   if (p.tiles >= (int64_t)1 << 31) return fail(NBTC_ERR_UNSUPPORTED, "more than 2^31 tiles");
   int W, slots;
   tc_shape_of(ctx, form, W, slots);
-  p.tmem_a = ctx->tc_tmem_a ? 1 : 0;
+  p.tmem_a = ctx->tc_tmem_a || !packed ? 1 : 0;
   int64_t grid = (p.tiles + W * slots - 1) / (W * slots);
   if (grid > ctx->sm_count) grid = ctx->sm_count;
   p.per_cta = (p.tiles + grid - 1) / grid;

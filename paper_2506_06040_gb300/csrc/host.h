@@ -14,7 +14,6 @@ struct nbtc_context {
   long long wait_budget = 0;       // spins per bounded device wait (0 = default, -1 = give up at once)
   int tc_groups = 4;               // warpgroups per CTA of the tensor-core decode (3 or 4)
   int tc_tmem_a = 1;               // MMA A operands in TMEM (one slot per warpgroup; 0: shared memory)
-  int fp32_groups = 2;             // independent thread groups per CTA of the FP32 wide decode (1 or 2)
   int check_plant = 0;             // checked build, tests only: offset added to gather indices
   int train_tc = 1;                // training steps with pre-gathered samples on tensor cores (0: SIMT)
 };
@@ -59,8 +58,10 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 
 // Kernel launchers (one per translation unit).
 nbtc_status launch_bc1_decode(nbtc_context* ctx, const LevelView& v, uint8_t* out, cudaStream_t s);
-nbtc_status launch_decode_fp32(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp,
+nbtc_status launch_decode_fp32(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, bool host_out,
                                cudaStream_t s);
+nbtc_status launch_decode_fp32_tc(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, bool host_out,
+                                  cudaStream_t s);
 nbtc_status tc_packed_bytes(const nbtc_mlp* mlp, int precision, size_t* bytes);
 nbtc_status launch_pack_mlp(nbtc_context* ctx, const nbtc_mlp* mlp, int precision, const float* act_absmax,
                             void* packed, size_t packed_bytes, cudaStream_t s);

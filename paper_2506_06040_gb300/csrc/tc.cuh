@@ -93,11 +93,15 @@ struct WorkChunk {
   int pad;
 };
 
-enum TcMode { kModeSingle = 0, kModeBatch = 1 };
+enum TcMode { kModeSingle = 0, kModeBatch = 1, kModeInPlace = 2 };
 
 struct TcArgs {
   DecodeArgs d;
   const void* packed;
+  const float* W;      // FP32 decodes (packed NULL): the MLP itself, laid out by each CTA
+  const float* B;
+  int hid;
+  int host_out;        // FP32 decodes: out is pinned host memory (plain stores)
   int nout;
   int footprint;       // 1: row-footprint feature stage
   int whole_rows;      // single material: every warp's 32 output rows exist and start on 16 bytes

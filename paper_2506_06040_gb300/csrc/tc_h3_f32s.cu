@@ -4,6 +4,7 @@
 namespace nbtc {
 
 nbtc_status launch_tc_h3_f32s(const TcArgs& p, int W, int slots, int grid, cudaStream_t s) {
+  if (p.mode == kModeInPlace) return launch_tc_w<3, kF32Split, 4, kModeInPlace, 1, true>(p, grid, s);  // FP32 decodes
   if (p.tmem_a && W == 4 && slots == 1)  // A operands in TMEM
     return launch_tc_w<3, kF32Split, 4, kModeSingle, 1, true>(p, grid, s);
   if (W == 4 && slots == 1) return launch_tc_w<3, kF32Split, 4, kModeSingle, 1>(p, grid, s);

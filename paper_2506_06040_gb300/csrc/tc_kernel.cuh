@@ -21,6 +21,7 @@
 
 #include <cstring>
 
+#include "f32s_pack.cuh"
 #include "features.cuh"
 #include "host.h"
 #include "sm100.cuh"
@@ -77,6 +78,31 @@ __device__ __forceinline__ void put_staged(unsigned char* dst, uint32_t stage, u
       if constexpr (UNIT == 2) *reinterpret_cast<uint16_t*>(g0 + at) = lds16(stage + at);
       else *reinterpret_cast<uint32_t*>(g0 + at) = lds32(stage + at);
     }
+  }
+}
+
+// One texel of an FP32 decode in plain FP32 multiply-adds, as the FFMA kernels
+// take it (bias first, inputs in order, ReLU dropping NaN): for MLPs that no FP16
+// scale can hold (weights that are not finite) and texels whose coordinate is NaN.
+// Slow, and out of line: neither occurs in a decode that means anything.
+static __device__ __noinline__ void fp32_texel(const DecodeArgs& d, const float* __restrict__ W, const float* __restrict__ B,
+                                        int nhid, int hid, int nout, int64_t tex, float* __restrict__ out) {
+  float x[12], h[2][kHid];
+  direct_features(d, tex, x);
+  for (int k = 0; k < 12; ++k) h[1][k] = x[k];
+  int in = 12;
+  for (int l = 0; l <= nhid; ++l) {
+    const int o = l == nhid ? nout : hid;
+    const float* from = h[(l + 1) & 1];
+    for (int r = 0; r < o; ++r) {
+      float s = B[r];
+      for (int k = 0; k < in; ++k) s = fmaf(from[k], W[r * in + k], s);
+      if (l == nhid) out[r] = s;
+      else h[l & 1][r] = fmaxf(s, 0.f);
+    }
+    W += in * o;
+    B += o;
+    in = o;
   }
 }
 
@@ -156,7 +182,8 @@ __host__ __device__ inline TcSmem tc_smem(const TcLayout& L, int W, int NSL, boo
 // Every thread keeps its whole schedule whatever happens -- after a timed-out
 // wait it stops waiting but still makes every arrival -- so both barrier kinds
 // always complete and the kernel always terminates.
-// MODE kModeSingle: one material whose views are kernel parameters; kModeBatch:
+// MODE kModeSingle: one material whose views are kernel parameters; kModeInPlace:
+// the same with the MLP laid out by each CTA (FP32 decodes); kModeBatch:
 // chunks of many materials (and frame tiles) whose views live in shared memory.
 template <int NHID, int FORM, int W, int MODE, int NSL, bool TA = false>
 __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
@@ -235,6 +262,9 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
     __syncthreads();
     tc_fence_after();
   }
+  // FP32 decodes bring no packed image: each CTA lays the MLP out in its shared memory
+  constexpr bool kInPlace = MODE == kModeInPlace;
+  static_assert(!kInPlace || (FORM == kF32Split && TA), "FP32 decodes: the FP32-accurate form on TMEM operands");
   bool failed = false;
   uint32_t wph = 0;  // phase of the weight barrier
 
@@ -252,7 +282,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
     // ---- take the next chunk (thread 0), load its material's MLP if it changed
     if (tid == 0) {
       int valid = 0, reload = 0;
-      if (MODE == kModeSingle) {
+      if (MODE != kModeBatch) {
         if (first_chunk) {
           const int64_t b = (int64_t)blockIdx.x * p.per_cta;
           const int64_t e = b + p.per_cta < p.tiles ? b + p.per_cta : p.tiles;
@@ -277,7 +307,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           valid = 1;
         }
       }
-      if (valid && reload) {
+      if (valid && reload && !kInPlace) {
         mbar_expect_tx(wbar, (uint32_t)L.bytes());
         bulk_g2s(sbase, work.m.packed, (uint32_t)L.bytes(), wbar);
       }
@@ -293,14 +323,36 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
         uint32_t* to = reinterpret_cast<uint32_t*>(&work.m);
         for (int i = tid; i < (int)(sizeof(MatDev) / 4); i += W * kTile + 32 * W) to[i] = __ldg(from + i);
       }
-      // always waited (fixed budget), also after a timed-out D-ready wait: the
-      // copy must land before the MMAs read the image and before the CTA exits
-      if (!mbar_wait_bounded(wbar, wph, kDrainBudget)) failed = true;
-      wph ^= 1u;
+      if constexpr (kInPlace) {
+        constexpr int nt = W * kTile + 32 * W;
+        F32sScratch& sc = *reinterpret_cast<F32sScratch*>(smem + S.stage);  // the stages are not in use yet
+        static_assert(sizeof(F32sScratch) <= W * 4 * stage_bytes(FORM), "scales in the output stages");
+        for (int i = tid; i < L.bytes() / 16; i += nt) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0u, 0u, 0u, 0u);
+        f32s_scales(p.W, p.B, NHID, p.hid, p.nout, tid, nt, sc);
+        if (sc.bad) {  // no scaled image: texel by texel
+          float* o = reinterpret_cast<float*>(p.d.out);
+          for (int64_t i = tid; i < (int64_t)work.c.count * kTile; i += nt) {
+            const int row = (int)(i % kTile);
+            const WarpRows wr = warp_rows(p.d, p.hdiv, p.footprint != 0, work.c.first + i / kTile, row / 32);
+            if ((row & 31) < wr.live) {
+              const int64_t tex = wr.first + (row & 31);
+              fp32_texel(p.d, p.W, p.B, NHID, p.hid, p.nout, tex, o + tex * p.nout);
+            }
+          }
+          break;
+        }
+        f32s_pack(smem, L, p.W, p.B, p.hid, p.nout, tid, nt, sc);
+        fence_proxy_async_smem();
+      } else {
+        // always waited (fixed budget), also after a timed-out D-ready wait: the
+        // copy must land before the MMAs read the image and before the CTA exits
+        if (!mbar_wait_bounded(wbar, wph, kDrainBudget)) failed = true;
+        wph ^= 1u;
+      }
     }
     failed = __syncthreads_or(failed);
     const bool grid_chunk = work.c.kind == kChunkGrid;
-    const bool footprint = MODE == kModeSingle ? p.footprint != 0 : grid_chunk;
+    const bool footprint = MODE != kModeBatch ? p.footprint != 0 : grid_chunk;
     const int64_t range_end = work.c.count;   // tiles are numbered 0 .. count-1 inside the chunk
 
     // Schedule.  Warpgroup g decodes the contiguous tile range [g_begin, g_end)
@@ -375,9 +427,9 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
                 } else if (l == 0) {
                   if constexpr (F16S) {
                     // A0: hi [x 1 000] in the 8 columns at ah, lo [x 1 000] at al
-                    mma_f16_ts(d, ah, dsc(hi_w1, lo_w1), ID_HID, 0);       // hi x . hi W + hi b
-                    mma_f16_ts(d, al, dsc(hi_w1, lo_w1 + 16), ID_HID, 1);  // lo x . hi W + lo b
+                    mma_f16_ts(d, al, dsc(hi_w1, lo_w1 + 16), ID_HID, 0);  // lo x . hi W + lo b
                     mma_f16_ts(d, ah, dsc(hi_w1, lo_w1 + 32), ID_HID, 1);  // hi x . lo W
+                    mma_f16_ts(d, ah, dsc(hi_w1, lo_w1), ID_HID, 1);       // hi x . hi W + hi b
                   } else {
                     mma_f16_ts(d, ah, dsc(hi_w1, lo_w1), ID_HID, 0);       // [x 1 0 0 0] . [W b 0 0 0]
                   }
@@ -387,27 +439,31 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
                   const uint32_t lo_b = lo(sbase + (last ? L.off_wo() : L.off_wh(l - 1)), 16);
                   const uint32_t lo_bt = lo(sbase + (last ? L.off_bto() : L.off_bth(l - 1)), 128);
                   const uint32_t db = (uint32_t)(last ? L.wo_part() : L.wh_part()) >> 4;  // lo W, 16-byte units
+                  // split: the small products first, while the (truncating)
+                  // accumulator is small, then hi.hi (FP32-accurate 12-64-64-9: 4.8e-7
+                  // from FP64 in 2-norm with each chunk's three together, 2.2e-7 so)
                   if constexpr (kOnesT)
                     mma_f16_ts(d, tmem_base + kOnesCol, dsc(hi_int, lo_bt), id, 0);
                   else
                     mma_f16(d, dsc(hi_int, lo_ones), dsc(hi_int, lo_bt), id, 0);
+                  if constexpr (F16S) {
 #pragma unroll
-                  for (int kk = 0; kk < 4; ++kk) {
-                    mma_f16_ts(d, ah + 8 * kk, dsc(hi_w, lo_b + 2 * kk), id, 1);
-                    if constexpr (F16S) {
+                    for (int kk = 0; kk < 4; ++kk) {
                       mma_f16_ts(d, al + 8 * kk, dsc(hi_w, lo_b + 2 * kk), id, 1);
                       mma_f16_ts(d, ah + 8 * kk, dsc(hi_w, lo_b + db + 2 * kk), id, 1);
                     }
                   }
+#pragma unroll
+                  for (int kk = 0; kk < 4; ++kk) mma_f16_ts(d, ah + 8 * kk, dsc(hi_w, lo_b + 2 * kk), id, 1);
                 }
               } else if (l == 0) {
                 // K chunks of 32 bytes (16 FP16 / 32 E4M3), 256 bytes apart in
                 // the no-swizzle layout
                 const uint32_t la = lo(slot + S.a0, 128);
                 if constexpr (F16S) {
-                  mma_f16(d, dsc(hi_a0, la), dsc(hi_w1, lo_w1), ID_HID, 0);                // hi x . hi W + hi b
-                  mma_f16(d, dsc(hi_a0, la + 16), dsc(hi_w1, lo_w1 + 16), ID_HID, 1);      // lo x . hi W + lo b
+                  mma_f16(d, dsc(hi_a0, la + 16), dsc(hi_w1, lo_w1 + 16), ID_HID, 0);      // lo x . hi W + lo b
                   mma_f16(d, dsc(hi_a0, la), dsc(hi_w1, lo_w1 + 32), ID_HID, 1);           // hi x . lo W
+                  mma_f16(d, dsc(hi_a0, la), dsc(hi_w1, lo_w1), ID_HID, 1);                // hi x . hi W + hi b
                 } else if constexpr (FORM == kF8Split) {
                   mma_f8(d, dsc(hi_a0, la), dsc(hi_w1, lo_w1), ID_HID, 0);                 // [hi x | lo x] . hi W
                   mma_f8(d, dsc(hi_a0, la), dsc(hi_w1, lo_w1 + 16), ID_HID, 1);            // [hi x | lo x] . [lo W | 0]
@@ -436,14 +492,16 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
                 } else {
                   const uint32_t lo_bt = lo(sbase + (last ? L.off_bto() : L.off_bth(l - 1)), 128);
                   mma_f16(d, dsc(hi_int, lo_ones), dsc(hi_int, lo_bt), id, 0);
+                  if constexpr (SPLIT) {
 #pragma unroll
-                  for (int kk = 0; kk < 4; ++kk) {
-                    mma_f16(d, dsc(hi_w, lo_a + 2 * kk), dsc(hi_w, lo_b + 2 * kk), id, 1);
-                    if constexpr (SPLIT) {
+                    for (int kk = 0; kk < 4; ++kk) {
                       mma_f16(d, dsc(hi_w, lo_a + da + 2 * kk), dsc(hi_w, lo_b + 2 * kk), id, 1);
                       mma_f16(d, dsc(hi_w, lo_a + 2 * kk), dsc(hi_w, lo_b + db + 2 * kk), id, 1);
                     }
                   }
+#pragma unroll
+                  for (int kk = 0; kk < 4; ++kk)
+                    mma_f16(d, dsc(hi_w, lo_a + 2 * kk), dsc(hi_w, lo_b + 2 * kk), id, 1);
                 }
               }
               mma_commit(dbar0 + q * 8);
@@ -473,14 +531,17 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
       const uint32_t stage_s = sbase + S.stage + warp * stage_bytes(FORM);
       const float* bias = reinterpret_cast<const float*>(smem + L.off_bias());
       const float* alpha = reinterpret_cast<const float*>(smem + L.off_alpha());
-      const DecodeArgs& D = MODE == kModeSingle ? p.d : work.m.d;
-      const FastDiv& hdiv = MODE == kModeSingle ? p.hdiv : work.m.hdiv;
+      const DecodeArgs& D = MODE != kModeBatch ? p.d : work.m.d;
+      const FastDiv& hdiv = MODE != kModeBatch ? p.hdiv : work.m.hdiv;
       const int nout = work.m.nout;
       const bool whole_rows = p.whole_rows != 0;
       const int64_t g_begin = min((int64_t)wg * per_wg, range_end);
       const int64_t g_end = min(g_begin + per_wg, range_end);
       StripCache cache;
       strip_reset(cache);
+      // FP32 decodes of a uv list: this thread's texel has a NaN coordinate (its
+      // features are NaN; the FFMA kernels' ReLU drops that, the conversions keep it)
+      bool nan_cur[kSlots] = {}, nan_next = false;
       uint32_t next_a0[16];  // TA: the next tile's A0, computed during the output layer's MMAs
 
       // the 12 features of this thread's texel of tile T (full decode)
@@ -494,6 +555,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
         } else {
           const int64_t tex = (work.c.first + T) * kTile + gt;
           direct_features(D, tex < D.n ? tex : D.n - 1, f);
+          if (kInPlace) nan_next = f[0] != f[0];
         }
       };
       // TA: a tile's A0 row as it goes into TMEM (8 columns; split FP16: hi in
@@ -538,7 +600,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
       // the packed A0 row of this thread's row of tile T: from the features of its
       // texel, or (frame chunks, FP16 only) the row the feature pass left for its pixel px
       auto tile_row = [&](int64_t T, int px, uint32_t (&av)[16]) {
-        if (MODE == kModeSingle || grid_chunk) {
+        if (MODE != kModeBatch || grid_chunk) {
           float f[12];
           tile_features(T, f);
           pack_a0(f, av);
@@ -573,6 +635,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           uint32_t av[16];
           tile_row(T, cur_px[s], av);
           if constexpr (TA) {
+            if (kInPlace) nan_cur[s] = nan_next;
             store_a0(s, av);
             return;
           }
@@ -585,6 +648,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
         }
         float f[12];
         tile_features(T, f);
+        if (kInPlace) nan_cur[s] = nan_next;
         if constexpr (F16S) {
           uint32_t h[6], r[6];
 #pragma unroll
@@ -823,11 +887,41 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           if (odd && even_n) sts16(row + 2u * (uint32_t)(nout - 1), (uint16_t)last);
         };
         if constexpr (OUT32) {
-          // FP32 output (single-material grids and uv lists): the accumulator as is.
-          // The warp's live texels x nout floats are contiguous in the output:
-          // staged and written together
+          // back from the channels' power-of-two scales (f32s_pack.cuh)
+#pragma unroll
+          for (int k = 0; k < kMaxOut; k += 4) {
+            if (k >= nout) break;
+            const float4 m = *reinterpret_cast<const float4*>(b + k);
+            r[k] = __float_as_uint(__uint_as_float(r[k]) * m.x);
+            r[k + 1] = __float_as_uint(__uint_as_float(r[k + 1]) * m.y);
+            r[k + 2] = __float_as_uint(__uint_as_float(r[k + 2]) * m.z);
+            r[k + 3] = __float_as_uint(__uint_as_float(r[k + 3]) * m.w);
+          }
+          // FP32 output (single-material grids and uv lists).  The warp's live texels
+          // x nout floats are contiguous in the output: staged and written together
           const WarpRows wr = warp_rows(D, hdiv, footprint, work.c.first + T, wq);
-          if (whole_rows) {  // 128 nout bytes at a multiple of 16: one bulk copy
+          if (kInPlace && !footprint && nan_cur[s]) {
+            float y[kMaxOut];
+            fp32_texel(p.d, p.W, p.B, NHID, p.hid, p.nout, min(wr.first + lane, p.d.n - 1), y);
+#pragma unroll
+            for (int k = 0; k < kMaxOut; ++k)
+              if (k < nout) r[k] = __float_as_uint(y[k]);
+          }
+          if (kInPlace && p.host_out) {  // pinned host memory: plain stores, 16 bytes a lane where rows are whole
+            if (wr.live > 0) {
+              __syncwarp();  // the stage has been read
+#pragma unroll
+              for (int k = 0; k < kMaxOut; ++k)
+                if (k < nout) sts32(stage_s + 4u * (uint32_t)(lane * nout + k), r[k]);
+              __syncwarp();
+              float* dst = reinterpret_cast<float*>(D.out) + wr.first * nout;
+              if (whole_rows) {
+                for (int i = lane; i < 8 * nout; i += 32) reinterpret_cast<float4*>(dst)[i] = lds128f(stage_s + 16u * i);
+              } else {
+                for (int i = lane; i < wr.live * nout; i += 32) dst[i] = __uint_as_float(lds32(stage_s + 4u * i));
+              }
+            }
+          } else if (whole_rows) {  // 128 nout bytes at a multiple of 16: one bulk copy
             if (lane == 0) bulk_wait_read0();
             __syncwarp();
 #pragma unroll
@@ -851,7 +945,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             __syncwarp();
             put_staged<4>(dst, stage_s, off, 4u * (uint32_t)(wr.live * nout), lane);
           }
-        } else if (MODE == kModeSingle || grid_chunk) {
+        } else if (MODE != kModeBatch || grid_chunk) {
           const WarpRows wr = warp_rows(D, hdiv, footprint, work.c.first + T, wq);
           if (MODE == kModeBatch || whole_rows) {  // 64 nout bytes at a multiple of 16: one bulk copy
             if (lane == 0) bulk_wait_read0();
@@ -950,6 +1044,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             } else {
               const bool more = base + s + kSlots < g_end;
               output_epilogue(s, base + s, TA && more);
+              if (kInPlace && TA) nan_cur[s] = nan_next;
               if (frame_chunk) {
                 cur_px[s] = next_px[s];
                 next_px[s] = pixel_of(base + s + 2 * kSlots);

@@ -252,3 +252,114 @@ def test_row_bands_equal_the_whole_grid(nb, ctx, dims):
     ctx.sync()
     with pytest.raises(nb.NbtcError):
         nb.decode(ctx, mat, grid=(gw, gh), rows=(590, 20))
+
+
+def _fp32_reference(material, x):
+    """The MLP in FP64 with the kernels' ReLU: fmax(v, 0), which drops NaN."""
+    with np.errstate(all="ignore"):
+        h = x
+        n = len(material.mlp.weights)
+        for l, (w, b) in enumerate(zip(material.mlp.weights, material.mlp.biases)):
+            h = h @ w.astype(np.float64).T + b.astype(np.float64)
+            if l + 1 < n:
+                h = np.fmax(h, 0.0)
+    return h
+
+
+def _grid_x(material, gw, gh):
+    idx = np.arange(gw * gh)
+    return oracle.decode.features_at(material, oracle.sample.grid_coord(idx % gw, gw).astype(np.float64),
+                                     oracle.sample.grid_coord(idx // gw, gh).astype(np.float64))
+
+
+@pytest.mark.parametrize("dims", [[12, 64, 9], [12, 64, 64, 5], [12, 64, 64, 64, 16]])
+@pytest.mark.parametrize("spread", [0, 8, 30])
+def test_width_64_any_scale_of_weights(nb, ctx, dims, spread):
+    """Hidden width 64 runs on split FP16 operands: neurons whose weights are scaled
+    by powers of two up to 2^+-spread (and their outgoing weights by the inverse)
+    leave the network the same function, far outside FP16's range, and layers with
+    gains beyond it; FP32 and FP32_TC stay at FP32 accuracy of the unscaled network."""
+    wl = synth.small_decode_workload(256, dims, seed=160 + len(dims) + spread)
+    mlp = wl.material.mlp
+    x = _grid_x(wl.material, 256, 24)
+    ref = _fp32_reference(wl.material, x)
+    rng = np.random.default_rng(spread)
+    for l in range(len(dims) - 2):
+        f = 2.0 ** rng.integers(-spread, spread + 1, dims[l + 1])
+        mlp.weights[l] = (mlp.weights[l] * f[:, None]).astype(np.float32)
+        mlp.biases[l] = (mlp.biases[l] * f).astype(np.float32)
+        mlp.weights[l + 1] = (mlp.weights[l + 1] / f[None, :]).astype(np.float32)
+    gain = 2.0 ** rng.integers(-spread, spread + 1, dims[-1])
+    mlp.weights[-1] = (mlp.weights[-1] * gain[:, None]).astype(np.float32)
+    mlp.biases[-1] = (mlp.biases[-1] * gain).astype(np.float32)
+    mat = nb.Material.from_synth(wl.material)
+    y = nb.decode(ctx, mat, grid=(256, 24))
+    z = nb.decode(ctx, mat, nb.FP32_TC, nb.pack_mlp(ctx, mat, nb.FP32_TC), grid=(256, 24))
+    ctx.sync()
+    assert max_abs(y.cpu().numpy().astype(np.float64) / gain, ref) <= TOL_FP32
+    assert torch.equal(y, z)
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan, 3e38])
+def test_width_64_weights_without_a_scale(nb, ctx, value):
+    """A weight no FP16 scale can hold: the decode takes plain FP32 arithmetic."""
+    wl = synth.small_decode_workload(256, [12, 64, 64, 9], seed=170)
+    wl.material.mlp.weights[1][7, 11] = value
+    wl.material.mlp.weights[0][3, 2] = value
+    wl.material.mlp.weights[2][:, 3] = 0.0   # the overflowed neurons only where they stay finite or NaN alike
+    wl.material.mlp.weights[2][:, 7] = 0.0
+    mat = nb.Material.from_synth(wl.material)
+    for kw in (dict(grid=(150, 9)), dict(uv=torch.from_numpy(synth.random_uv(9, 333)).cuda())):
+        y = nb.decode(ctx, mat, **kw)
+        ctx.sync()
+        x = _grid_x(wl.material, 150, 9) if "grid" in kw else oracle.decode.features_at(
+            wl.material, *(kw["uv"].cpu().numpy().astype(np.float64).T))
+        x = x.astype(np.float32)
+        with np.errstate(all="ignore"):  # plain FP32, inputs in order
+            h = x
+            for l, (w, b) in enumerate(zip(wl.material.mlp.weights, wl.material.mlp.biases)):
+                s = np.broadcast_to(b, (len(h), len(b))).astype(np.float32)
+                for k in range(w.shape[1]):
+                    s = (s.astype(np.float64) + h[:, k:k + 1].astype(np.float64) * w[:, k].astype(np.float64)).astype(np.float32)
+                h = np.fmax(s, np.float32(0)) if l < 2 else s
+        got = y.cpu().numpy()
+        assert np.array_equal(np.isnan(got), np.isnan(h)) and np.array_equal(np.isinf(got), np.isinf(h))
+        fin = np.isfinite(h)
+        assert np.all(np.abs(got[fin].astype(np.float64) - h[fin]) <= 1e-5 * np.maximum(1.0, np.abs(h[fin])))
+
+
+def test_width_64_nan_coordinates(nb, ctx):
+    """A NaN coordinate under wrap addressing gives NaN features, which the FP32 ReLU
+    drops: the texel decodes to the network of dead first-layer neurons, and its
+    neighbours are not touched."""
+    wl = synth.small_decode_workload(256, [12, 64, 64, 9], seed=171, address="wrap")
+    mat = nb.Material.from_synth(wl.material)
+    uv = synth.random_uv(10, 700)
+    clean = nb.decode(ctx, mat, uv=torch.from_numpy(uv).cuda())
+    bad = [0, 31, 128, 129, 500, 699]
+    uv[bad, 0] = np.nan
+    uv[129, 1] = np.inf
+    y = nb.decode(ctx, mat, uv=torch.from_numpy(uv).cuda())
+    ctx.sync()
+    m = wl.material.mlp
+    h = np.fmax(m.weights[1].astype(np.float64) @ np.zeros(64) + m.biases[1], 0.0)
+    want = m.weights[2].astype(np.float64) @ h + m.biases[2]
+    got = y.cpu().numpy().astype(np.float64)
+    assert np.abs(got[bad] - want).max() <= TOL_FP32
+    keep = np.setdiff1d(np.arange(700), bad)
+    assert torch.equal(y[keep], clean[keep])
+
+
+@pytest.mark.parametrize("gw,gh,nout", [(1500, 7, 9), (130, 20, 5), (256, 9, 16), (31, 5, 9)])
+def test_width_64_host_output_of_ragged_grids(nb, ctx, gw, gh, nout):
+    """Pinned host output (plain stores) holds the device output's bits."""
+    wl = synth.small_decode_workload(256, [12, 64, 64, nout], seed=172 + gw)
+    mat = nb.Material.from_synth(wl.material)
+    want = nb.decode(ctx, mat, grid=(gw, gh)).cpu()
+    off = 4 if nout % 4 else 1
+    host = torch.full((gw * gh + 2 * off, nout), 5.0).pin_memory()
+    out = host[off:off + gw * gh]
+    nb.decode(ctx, mat, grid=(gw, gh), out=out)
+    ctx.sync()
+    assert torch.equal(out, want)
+    assert bool((host[:off] == 5).all()) and bool((host[off + gw * gh:] == 5).all())
