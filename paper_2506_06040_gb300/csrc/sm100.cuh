@@ -216,6 +216,17 @@ __device__ __forceinline__ void mma_f8_ts(uint32_t d, uint32_t a, uint64_t b, ui
       : "memory");
 }
 
+// True in one lane of a converged warp (the same one every time).  The branch it
+// guards is known to run in one thread, so the operands of the MMAs in it go to
+// uniform registers directly: a stream of MMAs issues one per 10 .. 48 cycles, as the
+// tensor core takes them, where a branch on the lane number took at least 47 each
+// (measured: 128x64x16 with A in TMEM 32 against 47, 64x16x16 24 against 47).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.b32 %0, 1, 0, q;\n}" : "=r"(p));
+  return p != 0;
+}
+
 // Arrives once on `bar` when all tcgen05 operations this thread issued so far complete.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");

@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
     if (warp >= 4 * W) {
       // ---------------------------------------------------------- MMA warps
       // MMA warp m serves warpgroup m: it blocks in the hardware barrier (no
-      // polling) until the warpgroup has handed a slot over, then lane 0 issues
+      // polling) until the warpgroup has handed a slot over, then one lane issues
       // that layer's MMAs and commits them to the slot's D-ready mbarrier.
       // Descriptors are built once; per MMA only the 32-bit low word advances.
       const int m = warp - 4 * W;
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             if (s == 1 && !two) break;
             const int q = m * kSlots + s;
             named_bar_sync(bar_a(q), kTile + 32);
-            if (lane == 0) {
+            if (elect_one()) {
               tc_fence_after();
               const uint32_t d = tmem_base + (uint32_t)q * kHid;
               const uint32_t slot = sbase + S.slots + q * S.slot;
@@ -1066,7 +1066,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
   // Drain: the issuing lane of each MMA warp commits once more and waits for it
   // (drain budget), so that TMEM is released only after every MMA it issued has
   // completed -- also when a D-ready wait gave up and the warpgroup ran ahead.
-  if (warp >= 4 * W && lane == 0) {
+  if (warp >= 4 * W && elect_one()) {
     const uint32_t db = wbar + 8 + (warp - 4 * W) * 8;
     mma_commit(db);
     if (!mbar_wait_bounded(db, 0, kDrainBudget)) failed = true;
