@@ -21,6 +21,7 @@
 #include <string>
 
 #include "host.h"
+#include "sm100.cuh"
 
 namespace nbtc {
 
@@ -66,6 +67,17 @@ struct TrainDev {
 __device__ __forceinline__ void neumaier(float& s, float& e, float x) {
   const float t = s + x;
   e += (fabsf(s) >= fabsf(x)) ? ((s - t) + x) : ((x - t) + s);
+  s = t;
+}
+
+// (s, e) += x for a pair of sums, exact sum ~ s + e: the branch-free two-sum
+// (Knuth), every operation a packed pair.
+__device__ __forceinline__ void two_sum2(float2& s, float2& e, float2 x) {
+  const float2 m = make_float2(-1.f, -1.f);
+  const float2 t = __fadd2_rn(s, x);
+  const float2 z = __ffma2_rn(s, m, t);                                  // t - s
+  const float2 a = __ffma2_rn(__ffma2_rn(z, m, t), m, s), b = __ffma2_rn(z, m, x);  // s - (t - z), x - z
+  e = __fadd2_rn(e, __fadd2_rn(a, b));
   s = t;
 }
 
@@ -115,12 +127,6 @@ __device__ __forceinline__ void check_taps(Taps& T, int64_t n, const TrainDev& a
   (void)a;
 #endif
 }
-
-}  // namespace nbtc
-
-#include "train_tc.cuh"
-
-namespace nbtc {
 
 // Shared memory of k_train: weights in both orientations (forward products
 // read W^T rows, backward products read W rows, both as broadcast 128-bit
@@ -302,32 +308,42 @@ __device__ __forceinline__ void sample_target_ilp(const TrainDev& a, float u, fl
 // to a multiple of 4 when the mode reads a target).
 __host__ __device__ inline int gathered_floats(int C, bool target) { return kIn + (target ? 4 * ((C + 3) / 4) : 0); }
 
-// k_gather: one thread per sample (many warps per SM, so the scattered latent
-// and target taps of many samples are in flight at once) writes the sample's
-// features and target channels as one contiguous record of a.rs floats, read
-// back by k_train with 16-byte coalesced loads.  Same arithmetic as k_train's
-// own gather.
+// The pre-gathered record of sample i (a.rs floats at a.xt): its 12 features and,
+// with a target, its target channels.  Same arithmetic as k_train's own gather.
 template <bool LV, bool TV>
-__global__ void __launch_bounds__(256) k_gather(TrainDev a, float* __restrict__ xt, int with_target) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.batch; i += (int64_t)gridDim.x * blockDim.x) {
-    const float2 uv = __ldg(reinterpret_cast<const float2*>(a.uv) + i);
-    float f[kIn];
-    sample_features<LV>(a, uv.x, uv.y, f);
-    float4* r = reinterpret_cast<float4*>(xt + i * a.rs);
-    r[0] = make_float4(f[0], f[1], f[2], f[3]);
-    r[1] = make_float4(f[4], f[5], f[6], f[7]);
-    r[2] = make_float4(f[8], f[9], f[10], f[11]);
-    if (with_target) {
-      float tv[kCMax];
+__device__ __forceinline__ void gather_record(const TrainDev& a, int64_t i, bool with_target) {
+  const float2 uv = __ldg(reinterpret_cast<const float2*>(a.uv) + i);
+  float f[kIn];
+  sample_features<LV>(a, uv.x, uv.y, f);
+  float4* r = reinterpret_cast<float4*>(const_cast<float*>(a.xt) + i * a.rs);
+  r[0] = make_float4(f[0], f[1], f[2], f[3]);
+  r[1] = make_float4(f[4], f[5], f[6], f[7]);
+  r[2] = make_float4(f[8], f[9], f[10], f[11]);
+  if (with_target) {
+    float tv[kCMax];
 #pragma unroll
-      for (int c = 0; c < kCMax; ++c) tv[c] = 0.f;
-      sample_target_ilp<TV>(a, uv.x, uv.y, tv, 1);
+    for (int c = 0; c < kCMax; ++c) tv[c] = 0.f;
+    sample_target_ilp<TV>(a, uv.x, uv.y, tv, 1);
 #pragma unroll
-      for (int q = 0; q < kCMax / 4; ++q)
-        if (4 * q < a.C) r[3 + q] = make_float4(tv[4 * q], tv[4 * q + 1], tv[4 * q + 2], tv[4 * q + 3]);
-    }
+    for (int q = 0; q < kCMax / 4; ++q)
+      if (4 * q < a.C) r[3 + q] = make_float4(tv[4 * q], tv[4 * q + 1], tv[4 * q + 2], tv[4 * q + 3]);
   }
 }
+
+// k_gather: one thread per sample (many warps per SM, so the scattered latent
+// and target taps of many samples are in flight at once); the records are read
+// back by k_train with 16-byte coalesced loads.
+template <bool LV, bool TV>
+__global__ void __launch_bounds__(256) k_gather(TrainDev a, int with_target) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.batch; i += (int64_t)gridDim.x * blockDim.x)
+    gather_record<LV, TV>(a, i, with_target != 0);
+}
+
+}  // namespace nbtc
+
+#include "train_tc.cuh"
+
+namespace nbtc {
 
 // LV: latents and latent gradients hold 4 floats per texel (16-byte texel
 // loads and 16-byte gradient adds); TV: the target's texel stride is a multiple
@@ -914,29 +930,41 @@ static TrainDev make_dev(const nbtc_train_args* A, void* workspace) {
 }
 
 template <bool LV, bool TV>
-static nbtc_status launch_k_gather(nbtc_context* ctx, const TrainDev& d, float* xt, int with_target, cudaStream_t s) {
+static nbtc_status launch_k_gather(nbtc_context* ctx, const TrainDev& d, int with_target, cudaStream_t s) {
   int64_t g = (d.batch + 255) / 256;
   if (g > (int64_t)ctx->sm_count * 8) g = (int64_t)ctx->sm_count * 8;
-  k_gather<LV, TV><<<(int)g, 256, 0, s>>>(d, xt, with_target);
+  k_gather<LV, TV><<<(int)g, 256, 0, s>>>(d, with_target);
   return cuda_check(cudaGetLastError(), "launch k_gather");
 }
 
-// Pre-gathers the batch's samples into the workspace when it has room for them.
-static nbtc_status pre_gather(nbtc_context* ctx, const nbtc_train_args* A, TrainDev& d, int grid, bool target,
-                              void* workspace, size_t workspace_bytes, cudaStream_t s) {
+// Whether the target is read 16 bytes at a time.
+static bool target_vec(const TrainDev& d) { return d.ts % 4 == 0 && aligned(d.target, 16); }
+
+// Points d at the samples' records when the workspace has room for them.
+static bool record_space(const nbtc_train_args* A, TrainDev& d, int grid, bool target, void* workspace,
+                         size_t workspace_bytes) {
   const int rs = gathered_floats(d.C, target);
   const size_t off = partials_bytes(grid);
-  if (A->batch <= 0 || workspace_bytes < off + (size_t)A->batch * rs * sizeof(float)) return NBTC_OK;
-  float* xt = reinterpret_cast<float*>(static_cast<char*>(workspace) + off);
+  if (A->batch <= 0 || workspace_bytes < off + (size_t)A->batch * rs * sizeof(float)) return false;
   d.rs = rs;
-  const bool lv = latent_stride(A) == 4, tv = target && d.ts % 4 == 0 && aligned(d.target, 16);
-  nbtc_status st = lv ? (tv ? launch_k_gather<true, true>(ctx, d, xt, target, s)
-                            : launch_k_gather<true, false>(ctx, d, xt, target, s))
-                      : (tv ? launch_k_gather<false, true>(ctx, d, xt, target, s)
-                            : launch_k_gather<false, false>(ctx, d, xt, target, s));
+  d.xt = reinterpret_cast<float*>(static_cast<char*>(workspace) + off);
+  return true;
+}
+
+// Gathers the batch's samples into their records.
+static nbtc_status pre_gather(nbtc_context* ctx, const nbtc_train_args* A, const TrainDev& d, bool target, cudaStream_t s) {
+  const bool lv = latent_stride(A) == 4, tv = target && target_vec(d);
+  return lv ? (tv ? launch_k_gather<true, true>(ctx, d, target, s) : launch_k_gather<true, false>(ctx, d, target, s))
+            : (tv ? launch_k_gather<false, true>(ctx, d, target, s) : launch_k_gather<false, false>(ctx, d, target, s));
+}
+
+template <bool LV, int CP>
+static nbtc_status launch_train_tc(const TrainDev& d, int grid, cudaStream_t s) {
+  nbtc_status st = cuda_check(cudaFuncSetAttribute(k_train_tc<LV, CP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   ttc::kSmem), "smem attr");
   if (st) return st;
-  d.xt = xt;
-  return NBTC_OK;
+  k_train_tc<LV, CP><<<grid, ttc::kThreads, ttc::kSmem, s>>>(d);
+  return cuda_check(cudaGetLastError(), "launch k_train_tc");
 }
 
 template <int MODE, bool LV, bool TV>
@@ -955,7 +983,7 @@ template <int MODE>
 static nbtc_status launch_train_kernel(const nbtc_train_args* A, const TrainDev& d, int grid, cudaStream_t s) {
   const bool lv = latent_stride(A) == 4;
   if constexpr (MODE == kModeTrain) {
-    const bool tv = d.ts % 4 == 0 && aligned(d.target, 16);
+    const bool tv = target_vec(d);
     if (lv) return tv ? launch_k_train<MODE, true, true>(d, grid, s) : launch_k_train<MODE, true, false>(d, grid, s);
     return tv ? launch_k_train<MODE, false, true>(d, grid, s) : launch_k_train<MODE, false, false>(d, grid, s);
   } else {
@@ -1001,19 +1029,19 @@ nbtc_status train_step_impl(nbtc_context* ctx, const nbtc_train_args* A, float* 
   if (loss && (st = need_readable(loss, "loss"))) return st;
   if (mode == kModeBwd && dy && (st = need_readable(dy, "dy"))) return st;
   if ((st = zero_latent_grads(ctx, A, s))) return st;
-  if ((st = pre_gather(ctx, A, d, grid, mode == kModeTrain, workspace, workspace_bytes, s))) return st;
+  // samples are gathered first where their records fit the workspace, and the step
+  // then runs on the tensor cores; otherwise the SIMT kernel gathers inside
+  const bool records = record_space(A, d, grid, mode == kModeTrain, workspace, workspace_bytes);
+  const bool tc = records && mode == kModeTrain && ctx->train_tc;
+  if (records && (st = pre_gather(ctx, A, d, mode == kModeTrain, s))) return st;
   if (mode == kModeBwd) {
     if (!dy && A->batch > 0) return fail(NBTC_ERR_INVALID_ARG, "dy is NULL");
     d.dy = dy;
     if ((st = launch_train_kernel<kModeBwd>(A, d, grid, s))) return st;
-  } else if (d.xt && ctx->train_tc) {
-    // pre-gathered records: the tensor-core kernel (two 128-sample warpgroups per CTA)
-    auto kern = latent_stride(A) == 4 ? k_train_tc<true> : k_train_tc<false>;
-    if ((st = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ttc::kSmem),
-                         "smem attr")))
-      return st;
-    kern<<<grid, ttc::kWG * 160, ttc::kSmem, s>>>(d);
-    if ((st = cuda_check(cudaGetLastError(), "launch k_train_tc"))) return st;
+  } else if (tc) {  // two 128-sample warpgroups per CTA
+    if (latent_stride(A) == 4) st = d.C <= 12 ? launch_train_tc<true, 12>(d, grid, s) : launch_train_tc<true, 16>(d, grid, s);
+    else st = d.C <= 12 ? launch_train_tc<false, 12>(d, grid, s) : launch_train_tc<false, 16>(d, grid, s);
+    if (st) return st;
   } else {
     if ((st = launch_train_kernel<kModeTrain>(A, d, grid, s))) return st;
   }
