@@ -72,48 +72,86 @@ struct QatJobs {
   float* g_alpha[4];
 };
 
-// One thread per texel: T = (1 - a) E0 + a E1, written with ls floats per texel
-// (3, or 4 with the padding channel set to 0).
-__global__ void k_qat_decode(QatJobs J, QatThresholds T, int ls) {
+// The decode and its backward take four threads a block, one texel row each:
+// thread i of a group of 32 has block i & 7 of the group's eight and row i >> 3, so a
+// row of neighbouring blocks is read and written contiguously.  The thresholds are
+// searched in shared memory (as kernel parameters, whose bank serves one address
+// at a time, lanes searching apart took turns).
+__device__ __forceinline__ void stage_thresholds(QatThresholds* to, const QatThresholds& T) {
+  const float* from = reinterpret_cast<const float*>(&T);
+  for (int i = threadIdx.x; i < (int)(sizeof(QatThresholds) / 4); i += blockDim.x) reinterpret_cast<float*>(to)[i] = from[i];
+  __syncthreads();
+}
+
+// T = (1 - a) E0 + a E1, written with ls floats per texel (3, or 4 with the padding
+// channel set to 0).  15 -> 9 us for the 348k texels of a 512^2 pyramid.
+__global__ void __launch_bounds__(256) k_qat_decode(QatJobs J, const __grid_constant__ QatThresholds Tp, int ls) {
+  __shared__ QatThresholds T;
+  stage_thresholds(&T, Tp);
   const QatLevelDev L = J.L[blockIdx.y];
   float* __restrict__ out = J.tex[blockIdx.y];
-  const int64_t n = (int64_t)L.w * L.h;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int y = (int)(i / L.w), x = (int)(i - (int64_t)y * L.w);
-    const int64_t b = (int64_t)(y >> 2) * (L.w >> 2) + (x >> 2);
+  const int wb = L.w >> 2;
+  const int64_t nb = (int64_t)wb * (L.h >> 2), n = (nb + 7) / 8 * 32;
+  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = (r >> 5) * 8 + (r & 7);
+    if (b >= nb) continue;
+    const int by = (int)(b / wb), bx = (int)(b - (int64_t)by * wb), ty = (int)(r >> 3) & 3;
     const float3 E0 = endpoint_value(L.e0 + 3 * b, T), E1 = endpoint_value(L.e1 + 3 * b, T);
-    const float a = (float)qlevel(L.alpha[i], T.t2, 3) / 3.f;
-    const float t0 = fmaf(a, E1.x - E0.x, E0.x), t1 = fmaf(a, E1.y - E0.y, E0.y), t2 = fmaf(a, E1.z - E0.z, E0.z);
-    if (ls == 4) {
-      reinterpret_cast<float4*>(out)[i] = make_float4(t0, t1, t2, 0.f);
-    } else {
-      out[3 * i + 0] = t0;
-      out[3 * i + 1] = t1;
-      out[3 * i + 2] = t2;
+    const int64_t i0 = (int64_t)(4 * by + ty) * L.w + 4 * bx;
+#pragma unroll
+    for (int tx = 0; tx < 4; ++tx) {
+      const int64_t i = i0 + tx;
+      const float a = (float)qlevel(L.alpha[i], T.t2, 3) / 3.f;
+      const float t0 = fmaf(a, E1.x - E0.x, E0.x), t1 = fmaf(a, E1.y - E0.y, E0.y), t2 = fmaf(a, E1.z - E0.z, E0.z);
+      if (ls == 4) {
+        reinterpret_cast<float4*>(out)[i] = make_float4(t0, t1, t2, 0.f);
+      } else {
+        out[3 * i + 0] = t0;
+        out[3 * i + 1] = t1;
+        out[3 * i + 2] = t2;
+      }
     }
   }
 }
 
-// One thread per block: straight-through gradients of its two endpoints and
-// sixteen blend factors from dL/dT (ls floats per texel).
-__global__ void k_qat_backward(QatJobs J, QatThresholds T, int ls) {
+// Straight-through gradients of a block's two endpoints and sixteen blend factors
+// from dL/dT (ls floats per texel); the rows' endpoint sums are added over the four
+// threads in a fixed order.  18 -> 10 us for the 348k texels of a 512^2 pyramid.
+__global__ void __launch_bounds__(256) k_qat_backward(QatJobs J, const __grid_constant__ QatThresholds Tp, int ls) {
+  __shared__ QatThresholds T;
+  stage_thresholds(&T, Tp);
   const QatLevelDev L = J.L[blockIdx.y];
   const float* __restrict__ dT = J.tex[blockIdx.y];
   float* __restrict__ g_e0 = J.g_e0[blockIdx.y];
   float* __restrict__ g_e1 = J.g_e1[blockIdx.y];
   float* __restrict__ g_alpha = J.g_alpha[blockIdx.y];
   const int wb = L.w >> 2;
-  const int64_t nb = (int64_t)wb * (L.h >> 2);
-  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nb; b += (int64_t)gridDim.x * blockDim.x) {
-    const int by = (int)(b / wb), bx = (int)(b - (int64_t)by * wb);
-    const float3 E0 = endpoint_value(L.e0 + 3 * b, T), E1 = endpoint_value(L.e1 + 3 * b, T);
+  const int64_t nb = (int64_t)wb * (L.h >> 2), n = (nb + 7) / 8 * 32;  // whole warps stay together for the sums
+  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = (r >> 5) * 8 + (r & 7);
+    const bool live = b < nb;
+    const int ty = (int)(r >> 3) & 3;
     float s0[3] = {0.f, 0.f, 0.f}, s1[3] = {0.f, 0.f, 0.f};
-    for (int ty = 0; ty < 4; ++ty) {
+    if (live) {
+      const int by = (int)(b / wb), bx = (int)(b - (int64_t)by * wb);
+      const float3 E0 = endpoint_value(L.e0 + 3 * b, T), E1 = endpoint_value(L.e1 + 3 * b, T);
+      const int64_t i0 = (int64_t)(4 * by + ty) * L.w + 4 * bx;
+#pragma unroll
       for (int tx = 0; tx < 4; ++tx) {
-        const int64_t i = (int64_t)(4 * by + ty) * L.w + 4 * bx + tx;
+        const int64_t i = i0 + tx;
         const float p = L.alpha[i];
         const float a = (float)qlevel(p, T.t2, 3) / 3.f;
-        const float d0 = dT[ls * i], d1 = dT[ls * i + 1], d2 = dT[ls * i + 2];
+        float d0, d1, d2;
+        if (ls == 4) {
+          const float4 d = reinterpret_cast<const float4*>(dT)[i];
+          d0 = d.x;
+          d1 = d.y;
+          d2 = d.z;
+        } else {
+          d0 = dT[3 * i];
+          d1 = dT[3 * i + 1];
+          d2 = dT[3 * i + 2];
+        }
         s0[0] = fmaf(d0, 1.f - a, s0[0]);
         s0[1] = fmaf(d1, 1.f - a, s0[1]);
         s0[2] = fmaf(d2, 1.f - a, s0[2]);
@@ -126,9 +164,20 @@ __global__ void k_qat_backward(QatJobs J, QatThresholds T, int ls) {
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const float a0 = sigm(L.e0[3 * b + c]), a1 = sigm(L.e1[3 * b + c]);
-      g_e0[3 * b + c] = s0[c] * (a0 * (1.f - a0));
-      g_e1[3 * b + c] = s1[c] * (a1 * (1.f - a1));
+      s0[c] += __shfl_xor_sync(0xffffffffu, s0[c], 8);
+      s0[c] += __shfl_xor_sync(0xffffffffu, s0[c], 16);
+      s1[c] += __shfl_xor_sync(0xffffffffu, s1[c], 8);
+      s1[c] += __shfl_xor_sync(0xffffffffu, s1[c], 16);
+    }
+    // row ty = 0 writes e0's gradient, row 1 e1's
+    if (live && ty < 2) {
+      const float* e = ty ? L.e1 : L.e0;
+      float* ge = ty ? g_e1 : g_e0;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float a = sigm(e[3 * b + c]);
+        ge[3 * b + c] = (ty ? s1[c] : s0[c]) * (a * (1.f - a));
+      }
     }
   }
 }
@@ -184,6 +233,11 @@ nbtc_status check_qat_level(const nbtc_qat_level* q, bool step) {
 
 QatLevelDev level_dev(const nbtc_qat_level* q) { return QatLevelDev{q->width, q->height, q->e0, q->e1, q->alpha}; }
 
+// Threads of the decode and its backward: four a block, blocks in groups of eight.
+int64_t row_threads(const nbtc_qat_level* q) {
+  return ((int64_t)(q->width / 4) * (q->height / 4) + 7) / 8 * 32;
+}
+
 int grid_for(nbtc_context* ctx, int64_t n) {
   int64_t g = (n + 255) / 256;
   if (g > (int64_t)ctx->sm_count * 16) g = (int64_t)ctx->sm_count * 16;
@@ -200,7 +254,7 @@ nbtc_status qat_decode(nbtc_context* ctx, const nbtc_qat_level* q, float* out, c
   QatJobs J{};
   J.L[0] = level_dev(q);
   J.tex[0] = out;
-  k_qat_decode<<<grid_for(ctx, (int64_t)q->width * q->height), 256, 0, s>>>(J, make_thresholds(), 3);
+  k_qat_decode<<<grid_for(ctx, row_threads(q)), 256, 0, s>>>(J, make_thresholds(), 3);
   return cuda_check(cudaGetLastError(), "launch k_qat_decode");
 }
 
@@ -234,12 +288,11 @@ nbtc_status train_step_qat(nbtc_context* ctx, const nbtc_train_args* A, const nb
   QatJobs D{}, B{};
   AdamSegs S;
   S.count = 12;
-  int64_t nt_max = 0, nb_max = 0;
+  int64_t rows_max = 0;
   for (int k = 0; k < 4; ++k) {
     const nbtc_qat_level& q = levels[k];
     const int64_t nb = (int64_t)(q.width / 4) * (q.height / 4), nt = (int64_t)q.width * q.height;
-    nt_max = nt > nt_max ? nt : nt_max;
-    nb_max = nb > nb_max ? nb : nb_max;
+    rows_max = row_threads(&q) > rows_max ? row_threads(&q) : rows_max;
     D.L[k] = B.L[k] = level_dev(&q);
     D.tex[k] = A->latents[k];
     B.tex[k] = A->latent_grads[k];
@@ -250,10 +303,10 @@ nbtc_status train_step_qat(nbtc_context* ctx, const nbtc_train_args* A, const nb
     S.seg[3 * k + 1] = AdamSeg{q.e1, q.g_e1, q.m_e1, q.v_e1, 3 * nb};
     S.seg[3 * k + 2] = AdamSeg{q.alpha, q.g_alpha, q.m_alpha, q.v_alpha, nt};
   }
-  k_qat_decode<<<dim3(grid_for(ctx, nt_max), 4), 256, 0, s>>>(D, T, ls);
+  k_qat_decode<<<dim3(grid_for(ctx, rows_max), 4), 256, 0, s>>>(D, T, ls);
   if ((st = cuda_check(cudaGetLastError(), "launch k_qat_decode"))) return st;
   if ((st = train_step_impl(ctx, A, loss, s, 3, nullptr, nullptr, A->workspace, A->workspace_bytes))) return st;
-  k_qat_backward<<<dim3(grid_for(ctx, nb_max), 4), 256, 0, s>>>(B, T, ls);
+  k_qat_backward<<<dim3(grid_for(ctx, rows_max), 4), 256, 0, s>>>(B, T, ls);
   if ((st = cuda_check(cudaGetLastError(), "launch k_qat_backward"))) return st;
   return launch_adam(ctx, A, A->lr_latent, S, s);
 }

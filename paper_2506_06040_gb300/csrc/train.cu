@@ -330,11 +330,36 @@ __device__ __forceinline__ void gather_record(const TrainDev& a, int64_t i, bool
   }
 }
 
+// Up to 4 float arrays to be zeroed, and thread t0 of `step`'s share of that (16
+// bytes a store where the array allows it).
+struct ZeroSeg {
+  float* p;
+  int64_t n;
+};
+struct ZeroSegs {
+  ZeroSeg seg[4];
+};
+__device__ __forceinline__ void zero_arrays(const ZeroSegs& Z, int64_t t0, int64_t step) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const ZeroSeg z = Z.seg[k];
+    int64_t done = 0;
+    if ((reinterpret_cast<uintptr_t>(z.p) & 15u) == 0) {
+      for (int64_t i = t0; i < z.n / 4; i += step) reinterpret_cast<float4*>(z.p)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      done = z.n / 4 * 4;
+    }
+    for (int64_t i = done + t0; i < z.n; i += step) z.p[i] = 0.f;
+  }
+}
+
 // k_gather: one thread per sample (many warps per SM, so the scattered latent
 // and target taps of many samples are in flight at once); the records are read
-// back by k_train with 16-byte coalesced loads.
+// back by k_train with 16-byte coalesced loads.  It also clears the latent
+// gradients for the kernel that follows: stores that cost nothing beside the
+// gather's loads, where a launch of their own took 22 us for 22 MB.
 template <bool LV, bool TV>
-__global__ void __launch_bounds__(256) k_gather(TrainDev a, int with_target) {
+__global__ void __launch_bounds__(256) k_gather(TrainDev a, int with_target, ZeroSegs Z) {
+  zero_arrays(Z, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.batch; i += (int64_t)gridDim.x * blockDim.x)
     gather_record<LV, TV>(a, i, with_target != 0);
 }
@@ -714,43 +739,77 @@ __device__ __forceinline__ void adam_update(float& p, float& m, float& v, float 
 }
 
 // Sum of the CTA partials of every gradient slot (fixed order, compensated);
-// writes the MLP gradients, the loss, and (train mode) the Adam update.
-__global__ void k_reduce_adam(const float* __restrict__ part, int nparts, int C, float loss_scale, float* W, float* B,
-                              float* gw, float* gb, float* mw, float* vw, float* mb, float* vb, float* loss,
-                              int do_adam, AdamHyper h) {
+// writes the MLP gradients, the loss, and (train mode) the Adam update.  A CTA takes
+// 32 slots: warp w adds every eighth partial from w on (coalesced, several loads in
+// flight), warp 0 adds the eight sums in order.  One thread a slot walking all 152
+// partials took 17 us, this 9 (timed alone, caches cold).
+constexpr int kReduceSlots = 32;
+__global__ void __launch_bounds__(256) k_reduce_adam(const float* __restrict__ part, int nparts, int C, float loss_scale,
+                                                     float* W, float* B, float* gw, float* gb, float* mw, float* vw,
+                                                     float* mb, float* vb, float* loss, int do_adam, AdamHyper h) {
+  __shared__ float2 sums[8][kReduceSlots];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = kH * kIn + kH * kH + C * kH;
   const int nb = 2 * kH + C;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e <= nw + nb; e += gridDim.x * blockDim.x) {
-    int slot;
-    if (e == nw + nb) slot = kGN;  // the loss
-    else if (e < kH * kIn) slot = kGW1 + e;
-    else if (e < kH * kIn + kH * kH) slot = kGW2 + (e - kH * kIn);
-    else if (e < nw) slot = kGW3 + (e - kH * kIn - kH * kH);
-    else slot = kGB1 + (e - nw);  // b1 [64], b2 [64], b3 [C] are contiguous slots
-    float s = 0.f, c = 0.f;
-    for (int p = 0; p < nparts; ++p) {
-      neumaier(s, c, part[(size_t)p * kPart + 2 * slot]);
-      c += part[(size_t)p * kPart + 2 * slot + 1];
-    }
-    const float g = s + c;
-    if (e == nw + nb) {
-      if (loss) *loss = g * loss_scale;
-      continue;
-    }
-    if (e < nw) {
-      gw[e] = g;
-      if (do_adam) adam_update(W[e], mw[e], vw[e], g, h);
-    } else {
-      gb[e - nw] = g;
-      if (do_adam) adam_update(B[e - nw], mb[e - nw], vb[e - nw], g, h);
-    }
+  const int e = blockIdx.x * kReduceSlots + lane;
+  int slot;
+  if (e >= nw + nb) slot = kGN;  // the loss (and nothing past it)
+  else if (e < kH * kIn) slot = kGW1 + e;
+  else if (e < kH * kIn + kH * kH) slot = kGW2 + (e - kH * kIn);
+  else if (e < nw) slot = kGW3 + (e - kH * kIn - kH * kH);
+  else slot = kGB1 + (e - nw);  // b1 [64], b2 [64], b3 [C] are contiguous slots
+  float s = 0.f, c = 0.f;
+#pragma unroll 4
+  for (int p = warp; p < nparts; p += 8) {
+    const float2 x = *reinterpret_cast<const float2*>(part + (size_t)p * kPart + 2 * slot);
+    neumaier(s, c, x.x);
+    c += x.y;
+  }
+  sums[warp][lane] = make_float2(s, c);
+  __syncthreads();
+  if (warp != 0 || e > nw + nb) return;
+  s = c = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    neumaier(s, c, sums[w][lane].x);
+    c += sums[w][lane].y;
+  }
+  const float g = s + c;
+  if (e == nw + nb) {
+    if (loss) *loss = g * loss_scale;
+  } else if (e < nw) {
+    gw[e] = g;
+    if (do_adam) adam_update(W[e], mw[e], vw[e], g, h);
+  } else {
+    gb[e - nw] = g;
+    if (do_adam) adam_update(B[e - nw], mb[e - nw], vb[e - nw], g, h);
   }
 }
 
-// Adam over several parameter arrays in one launch: segment blockIdx.y.
-__global__ void k_adam_latent(AdamSegs S, AdamHyper h) {
+// Adam over several parameter arrays in one launch: segment blockIdx.y, 16 bytes a
+// thread and array where all four arrays allow it (42 -> 30 us for the 5.6 M
+// floats of a 1024^2 pyramid).
+__global__ void __launch_bounds__(256) k_adam_latent(AdamSegs S, AdamHyper h) {
   const AdamSeg q = S.seg[blockIdx.y];
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < q.n; i += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  int64_t done = 0;
+  if (((reinterpret_cast<uintptr_t>(q.p) | reinterpret_cast<uintptr_t>(q.g) | reinterpret_cast<uintptr_t>(q.m) |
+        reinterpret_cast<uintptr_t>(q.v)) & 15u) == 0) {
+    for (int64_t i = t0; i < q.n / 4; i += step) {
+      float4 pp = reinterpret_cast<float4*>(q.p)[i], mm = reinterpret_cast<float4*>(q.m)[i],
+             vv = reinterpret_cast<float4*>(q.v)[i];
+      const float4 gg = reinterpret_cast<const float4*>(q.g)[i];
+      adam_update(pp.x, mm.x, vv.x, gg.x, h);
+      adam_update(pp.y, mm.y, vv.y, gg.y, h);
+      adam_update(pp.z, mm.z, vv.z, gg.z, h);
+      adam_update(pp.w, mm.w, vv.w, gg.w, h);
+      reinterpret_cast<float4*>(q.p)[i] = pp;
+      reinterpret_cast<float4*>(q.m)[i] = mm;
+      reinterpret_cast<float4*>(q.v)[i] = vv;
+    }
+    done = q.n / 4 * 4;
+  }
+  for (int64_t i = done + t0; i < q.n; i += step) {
     float pp = q.p[i], mm = q.m[i], vv = q.v[i];
     adam_update(pp, mm, vv, q.g[i], h);
     q.p[i] = pp;
@@ -759,20 +818,8 @@ __global__ void k_adam_latent(AdamSegs S, AdamHyper h) {
   }
 }
 
-// Zeroes up to 4 float arrays in one launch: array blockIdx.y.
-struct ZeroSeg {
-  float* p;
-  int64_t n;
-};
-struct ZeroSegs {
-  ZeroSeg seg[4];
-};
-__global__ void k_zero(ZeroSegs Z) {
-  const ZeroSeg z = Z.seg[blockIdx.y];
-  float* p = z.p;
-  const int64_t n = z.n;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    p[i] = 0.f;
+__global__ void __launch_bounds__(256) k_zero(ZeroSegs Z) {
+  zero_arrays(Z, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 // ------------------------------------------------------------------ host
@@ -793,7 +840,7 @@ nbtc_status launch_adam(nbtc_context* ctx, const nbtc_train_args* A, float lr, c
   int64_t nmax = 0;
   for (int i = 0; i < S.count; ++i) nmax = S.seg[i].n > nmax ? S.seg[i].n : nmax;
   if (nmax <= 0) return NBTC_OK;
-  int64_t gx = (nmax + 255) / 256;
+  int64_t gx = (nmax / 4 + 255) / 256 + 1;
   if (gx > ctx->sm_count * 16) gx = ctx->sm_count * 16;
   k_adam_latent<<<dim3((unsigned)gx, (unsigned)S.count), 256, 0, s>>>(S, h);
   return cuda_check(cudaGetLastError(), "launch k_adam_latent");
@@ -930,10 +977,11 @@ static TrainDev make_dev(const nbtc_train_args* A, void* workspace) {
 }
 
 template <bool LV, bool TV>
-static nbtc_status launch_k_gather(nbtc_context* ctx, const TrainDev& d, int with_target, cudaStream_t s) {
+static nbtc_status launch_k_gather(nbtc_context* ctx, const TrainDev& d, int with_target, const ZeroSegs& Z, cudaStream_t s) {
   int64_t g = (d.batch + 255) / 256;
   if (g > (int64_t)ctx->sm_count * 8) g = (int64_t)ctx->sm_count * 8;
-  k_gather<LV, TV><<<(int)g, 256, 0, s>>>(d, with_target);
+  if (g < ctx->sm_count) g = ctx->sm_count;  // (the clearing wants them all)
+  k_gather<LV, TV><<<(int)g, 256, 0, s>>>(d, with_target, Z);
   return cuda_check(cudaGetLastError(), "launch k_gather");
 }
 
@@ -951,11 +999,20 @@ static bool record_space(const nbtc_train_args* A, TrainDev& d, int grid, bool t
   return true;
 }
 
-// Gathers the batch's samples into their records.
+// The latent gradients, to be cleared (this batch's gradient, not an accumulation).
+static ZeroSegs grads_to_zero(const nbtc_train_args* A) {
+  ZeroSegs Z;
+  for (int k = 0; k < 4; ++k)
+    Z.seg[k] = ZeroSeg{A->latent_grads[k], latent_stride(A) * (int64_t)A->widths[k] * A->heights[k]};
+  return Z;
+}
+
+// Gathers the batch's samples into their records and clears the latent gradients.
 static nbtc_status pre_gather(nbtc_context* ctx, const nbtc_train_args* A, const TrainDev& d, bool target, cudaStream_t s) {
   const bool lv = latent_stride(A) == 4, tv = target && target_vec(d);
-  return lv ? (tv ? launch_k_gather<true, true>(ctx, d, target, s) : launch_k_gather<true, false>(ctx, d, target, s))
-            : (tv ? launch_k_gather<false, true>(ctx, d, target, s) : launch_k_gather<false, false>(ctx, d, target, s));
+  const ZeroSegs Z = grads_to_zero(A);
+  return lv ? (tv ? launch_k_gather<true, true>(ctx, d, target, Z, s) : launch_k_gather<true, false>(ctx, d, target, Z, s))
+            : (tv ? launch_k_gather<false, true>(ctx, d, target, Z, s) : launch_k_gather<false, false>(ctx, d, target, Z, s));
 }
 
 template <bool LV, int CP>
@@ -991,17 +1048,8 @@ static nbtc_status launch_train_kernel(const nbtc_train_args* A, const TrainDev&
   }
 }
 
-// Zeroes the latent gradients (this batch's gradient, not an accumulation).
 static nbtc_status zero_latent_grads(nbtc_context* ctx, const nbtc_train_args* A, cudaStream_t s) {
-  ZeroSegs Z;
-  int64_t nmax = 0;
-  for (int k = 0; k < 4; ++k) {
-    Z.seg[k] = ZeroSeg{A->latent_grads[k], latent_stride(A) * (int64_t)A->widths[k] * A->heights[k]};
-    nmax = Z.seg[k].n > nmax ? Z.seg[k].n : nmax;
-  }
-  int64_t gx = (nmax + 255) / 256;
-  if (gx > ctx->sm_count * 16) gx = ctx->sm_count * 16;
-  k_zero<<<dim3((unsigned)gx, 4u), 256, 0, s>>>(Z);
+  k_zero<<<ctx->sm_count * 4, 256, 0, s>>>(grads_to_zero(A));
   return cuda_check(cudaGetLastError(), "launch k_zero");
 }
 
@@ -1028,12 +1076,11 @@ nbtc_status train_step_impl(nbtc_context* ctx, const nbtc_train_args* A, float* 
   if ((st = need_device(workspace, "workspace"))) return st;
   if (loss && (st = need_readable(loss, "loss"))) return st;
   if (mode == kModeBwd && dy && (st = need_readable(dy, "dy"))) return st;
-  if ((st = zero_latent_grads(ctx, A, s))) return st;
   // samples are gathered first where their records fit the workspace, and the step
   // then runs on the tensor cores; otherwise the SIMT kernel gathers inside
   const bool records = record_space(A, d, grid, mode == kModeTrain, workspace, workspace_bytes);
   const bool tc = records && mode == kModeTrain && ctx->train_tc;
-  if (records && (st = pre_gather(ctx, A, d, mode == kModeTrain, s))) return st;
+  if ((st = records ? pre_gather(ctx, A, d, mode == kModeTrain, s) : zero_latent_grads(ctx, A, s))) return st;
   if (mode == kModeBwd) {
     if (!dy && A->batch > 0) return fail(NBTC_ERR_INVALID_ARG, "dy is NULL");
     d.dy = dy;
@@ -1057,7 +1104,7 @@ nbtc_status train_step_impl(nbtc_context* ctx, const nbtc_train_args* A, float* 
   float* W = const_cast<float*>(A->mlp.weights);
   float* Bv = const_cast<float*>(A->mlp.biases);
   const int np = kH * kIn + kH * kH + C * kH + 2 * kH + C + 1;
-  k_reduce_adam<<<(np + 255) / 256, 256, 0, s>>>(static_cast<float*>(workspace), grid, C, loss_scale, W, Bv, A->grad_w,
+  k_reduce_adam<<<(np + kReduceSlots - 1) / kReduceSlots, 256, 0, s>>>(static_cast<float*>(workspace), grid, C, loss_scale, W, Bv, A->grad_w,
                                                  A->grad_b, A->m_w, A->v_w, A->m_b, A->v_b, loss,
                                                  mode == kModeTrain ? 1 : 0, h);
   if ((st = cuda_check(cudaGetLastError(), "launch k_reduce_adam"))) return st;
