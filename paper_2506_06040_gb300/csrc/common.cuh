@@ -114,48 +114,107 @@ __device__ __forceinline__ uint32_t fetch_texel(const LevelView& L, int x, int y
 
 // ---------------------------------------------------------------- sampling
 
-// Integer neighbours and fractional weight along one axis.  The texel
-// coordinate is t = u * n - 0.5 + shift; neighbours floor(t) and floor(t) + 1
-// are clamped to [0, n-1] or wrapped modulo n.
+// A coordinate as the samplers take it: under wrap addressing without its whole
+// periods (u - floor(u) is exact), so the texel coordinate keeps its fraction even
+// for tiled uv far from [0, 1).
+__device__ __forceinline__ float2 address_uv(float u, float v, bool wrap) {
+  return wrap ? make_float2(u - floorf(u), v - floorf(v)) : make_float2(u, v);
+}
+
+// Integer neighbours and fractional weight along one axis of an address_uv
+// coordinate.  The texel coordinate is t = u * n - 0.5 + shift; neighbours
+// floor(t) and floor(t) + 1 are clamped to [0, n-1] or wrapped modulo n.
+// HALF: the caller knows |shift| <= 1/2.
+template <bool HALF = false>
 __device__ __forceinline__ void axis_taps(float u, int n, float shift, bool wrap, int& i0, int& i1,
                                           float& f) {
-  // wrap: drop whole periods of u first (u - floor(u) is exact), so the texel
-  // coordinate keeps its fraction even for tiled uv far from [0, 1)
-  if (wrap) u -= floorf(u);
   float t = fmaf(u, (float)n, shift - 0.5f);
   if (!wrap) t = fminf(fmaxf(t, -1.0f), (float)n);  // outside this range clamping decides
   const float fl = floorf(t);
   f = t - fl;  // exact
   const int a = (int)fl;
-  if (wrap) {  // u in [0, 1] and |shift| <= 1/2: a in [-1, n], wrapped as an integer
-    i0 = a < 0 ? a + n : (a >= n ? a - n : a);
-    i1 = i0 + 1 >= n ? i0 + 1 - n : i0 + 1;
+  if (wrap) {
+    // u in [0, 1] and |shift| <= 1/2: a in [-1, n], wrapped by unsigned minima: x + n
+    // is the smaller one when x is negative, x - n when x has reached n
+    const uint32_t x = __viaddmin_u32((uint32_t)a, (uint32_t)n, (uint32_t)a);
+    i0 = (int)__viaddmin_u32(x, (uint32_t)-n, x);
+    i1 = (int)__viaddmin_u32((uint32_t)i0 + 1u, (uint32_t)-n, (uint32_t)i0 + 1u);
+    if (!HALF && fabsf(shift) > 0.5f) {  // further periods away
+      i0 = a % n < 0 ? a % n + n : a % n;
+      i1 = i0 + 1 == n ? 0 : i0 + 1;
+    }
   } else {
     i0 = min(max(a, 0), n - 1);
     i1 = min(max(a + 1, 0), n - 1);
   }
 }
 
-// Bilinear sample of one BC1 level at uv, FP32, channels in [0, 1].
+// ---- BC1 texels as FP32, for samples that decode at their taps.  A block's two
+// endpoints are widened with all three channels in 10-bit fields of one word; a
+// tap's palette numerators a0 e0 + a1 e1 + 1 are then two multiply-adds for the three
+// channels, and the rounded division by 3 (or 2) is one FP32 multiply-add each:
+// with F = 2^23 + num (the field under the exponent of 2^23),
+//   four colours   num = a0 e0 + a1 e1 + 1 <= 766:       RN(F / 3 + 9786709) = 2^23 + 2^22 + num div 3
+//   three colours  num = 2 (a0 e0 + a1 e1) + 1 <= 1021:  RN(F / 4 + 10485760) = 2^23 + 2^22 + (num + 1) div 4
+// (the second is (a0 e0 + a1 e1 + 1) div 2; both checked for every numerator on the
+// host against the integer form).  ~45 instructions a tap with its share of the
+// block, where the integer decode and conversion of bc1_texel took ~65.
+struct Bc1Block {
+  uint32_t e0, e1;  // endpoints: r | g << 10 | b << 20
+  uint32_t bits;    // 16 2-bit indices
+  uint32_t wt;      // byte i: endpoint weights a0 | a1 << 4 of index i
+  float scale, add;
+};
+
+__device__ __forceinline__ uint32_t widen565(uint32_t c) {
+  const uint32_t hi = ((c >> 8) & 0xF8u) | ((c << 7) & 0x3F000u) | ((c << 23) & 0xF800000u);
+  return hi | ((hi >> 5) & 0x700007u) | ((hi >> 6) & 0xC00u);
+}
+
+__device__ __forceinline__ Bc1Block bc1_block(uint64_t blk) {
+  const uint32_t lo = (uint32_t)blk, c0 = lo & 0xFFFFu, c1 = lo >> 16;
+  const bool four = c0 > c1;
+  Bc1Block b;
+  b.e0 = widen565(c0);
+  b.e1 = widen565(c1);
+  b.bits = (uint32_t)(blk >> 32);
+  b.wt = four ? 0x21123003u : 0x00224004u;
+  b.scale = four ? 1.0f / 3.0f : 0.25f;
+  b.add = four ? 9786709.0f : 10485760.0f;
+  return b;
+}
+
+constexpr float kTexelBase = 12582912.0f;  // 2^23 + 2^22
+
+// Texel (tx, ty) of a block: channels in 0..255 plus kTexelBase, exact.
+__device__ __forceinline__ float3 bc1_texel_f(const Bc1Block& b, int tx, int ty) {
+  const uint32_t w = b.wt >> (8u * ((b.bits >> (2 * (4 * ty + tx))) & 3u));
+  const uint32_t num = (w & 15u) * b.e0 + ((w >> 4) & 15u) * b.e1 + 0x00100401u;
+  auto ch = [&](uint32_t f) { return fmaf(__uint_as_float(0x4B000000u | f), b.scale, b.add); };
+  return make_float3(ch(num & 0x3FFu), ch((num >> 10) & 0x3FFu), ch(num >> 20));
+}
+
+// Bilinear sample of one BC1 level at an address_uv coordinate, FP32, channels in
+// [0, 1]: the horizontal blends of both rows as packed FP32 pairs, then the vertical one.
 __device__ __forceinline__ float3 sample_bilinear(const LevelView& L, float u, float v, bool wrap) {
   int x0, x1, y0, y1;
   float fx, fy;
   axis_taps(u, L.w, L.shift, wrap, x0, x1, fx);
   axis_taps(v, L.h, L.shift, wrap, y0, y1, fy);
-  const uint32_t t00 = fetch_texel(L, x0, y0), t10 = fetch_texel(L, x1, y0);
-  const uint32_t t01 = fetch_texel(L, x0, y1), t11 = fetch_texel(L, x1, y1);
-  const float w00 = (1.f - fx) * (1.f - fy), w10 = fx * (1.f - fy);
-  const float w01 = (1.f - fx) * fy, w11 = fx * fy;
-  float3 c;
+  const uint64_t b00 = __ldg(L.blocks + block_index(L, x0 >> 2, y0 >> 2)), b10 = __ldg(L.blocks + block_index(L, x1 >> 2, y0 >> 2));
+  const uint64_t b01 = __ldg(L.blocks + block_index(L, x0 >> 2, y1 >> 2)), b11 = __ldg(L.blocks + block_index(L, x1 >> 2, y1 >> 2));
+  const float3 t00 = bc1_texel_f(bc1_block(b00), x0 & 3, y0 & 3), t10 = bc1_texel_f(bc1_block(b10), x1 & 3, y0 & 3);
+  const float3 t01 = bc1_texel_f(bc1_block(b01), x0 & 3, y1 & 3), t11 = bc1_texel_f(bc1_block(b11), x1 & 3, y1 & 3);
   const float s = 1.0f / 255.0f;
-#define NBTC_CH(sh)                                                                          \
-  (s * (w00 * (float)((t00 >> sh) & 255u) + w10 * (float)((t10 >> sh) & 255u) +             \
-        w01 * (float)((t01 >> sh) & 255u) + w11 * (float)((t11 >> sh) & 255u)))
-  c.x = NBTC_CH(0);
-  c.y = NBTC_CH(8);
-  c.z = NBTC_CH(16);
-#undef NBTC_CH
-  return c;
+  auto blend = [&](float a0, float a1, float c0, float c1) {  // (top, bottom) left and right taps
+    const float2 l = make_float2(a0, a1), r = make_float2(c0, c1);
+    const float2 d = __fadd2_rn(r, make_float2(-l.x, -l.y));                    // exact
+    const float2 z = __fadd2_rn(l, make_float2(-kTexelBase, -kTexelBase));      // exact
+    const float2 q = __ffma2_rn(make_float2(fx, fx), d, z);
+    return s * fmaf(fy, q.y - q.x, q.x);
+  };
+  return make_float3(blend(t00.x, t01.x, t10.x, t11.x), blend(t00.y, t01.y, t10.y, t11.y),
+                     blend(t00.z, t01.z, t10.z, t11.z));
 }
 
 // Arguments shared by the decode kernels (passed by value).

@@ -431,7 +431,7 @@ __device__ __forceinline__ LevelView mip_view(const MatDev& M, int k, int m) {
 
 // Features of one texel sampled on its own (any uv).
 __device__ __forceinline__ void direct_features(const DecodeArgs& a, int64_t t, float (&feat)[12]) {
-  const float2 uv = texel_uv(a, t);
+  const float2 tuv = texel_uv(a, t), uv = address_uv(tuv.x, tuv.y, a.wrap);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const float3 c = sample_bilinear(a.lv[k], uv.x, uv.y, a.wrap);

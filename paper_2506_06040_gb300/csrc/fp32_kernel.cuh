@@ -157,10 +157,10 @@ __global__ void __launch_bounds__(256, 1)
     T x[kNin];
 #pragma unroll
     for (int q = 0; q < TPT; ++q) {
-      const float2 uv = texel_uv(a, tex[q]);
+      const float2 uv = texel_uv(a, tex[q]), auv = address_uv(uv.x, uv.y, a.wrap);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const float3 c = sample_bilinear(a.lv[k], uv.x, uv.y, a.wrap);
+        const float3 c = sample_bilinear(a.lv[k], auv.x, auv.y, a.wrap);
         VV::set(x[3 * k + 0], q, c.x);
         VV::set(x[3 * k + 1], q, c.y);
         VV::set(x[3 * k + 2], q, c.z);

@@ -48,8 +48,8 @@ __device__ __forceinline__ float3 sample_texels(const FrameFeatArgs& a, const Te
                                                 bool wrap) {
   int x0, x1, y0, y1;
   float fx, fy;
-  axis_taps(u, T.w, shift, wrap, x0, x1, fx);
-  axis_taps(v, T.h, shift, wrap, y0, y1, fy);
+  axis_taps<true>(u, T.w, shift, wrap, x0, x1, fx);
+  axis_taps<true>(v, T.h, shift, wrap, y0, y1, fy);
   const int r0 = y0 * T.w, r1 = y1 * T.w;
   const uint32_t t00 = texel_at(a, T, r0 + x0), t10 = texel_at(a, T, r0 + x1);
   const uint32_t t01 = texel_at(a, T, r1 + x0), t11 = texel_at(a, T, r1 + x1);
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(256) k_frame_features(FrameFeatArgs a) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-    auto probes = [&](float t, auto&& lower, auto&& upper) {
+    auto probes = [&](float t, bool wrap, auto&& lower, auto&& upper) {
 #pragma unroll 1
       for (int i = 1; i <= P.n; ++i) {
         float uu = uv.x, vv = uv.y;
@@ -141,7 +141,8 @@ __global__ void __launch_bounds__(256) k_frame_features(FrameFeatArgs a) {
           uu = fmaf(off, P.au, uu);
           vv = fmaf(off, P.av, vv);
         }
-        const float3 c0 = lower(uu, vv), c1 = upper(uu, vv);
+        const float2 at = address_uv(uu, vv, wrap);
+        const float3 c0 = lower(at.x, at.y), c1 = upper(at.x, at.y);
         s0 += fmaf(t, c1.x - c0.x, c0.x);
         s1 += fmaf(t, c1.y - c0.y, c0.y);
         s2 += fmaf(t, c1.z - c0.z, c0.z);
@@ -159,13 +160,13 @@ __global__ void __launch_bounds__(256) k_frame_features(FrameFeatArgs a) {
       const int4 g0 = __ldg(reinterpret_cast<const int4*>(L->mip + Q.m0));
       const int4 g1 = __ldg(reinterpret_cast<const int4*>(L->mip + Q.m1));
       const TexelView V0{base + (uint32_t)g0.x, g0.y, g0.z}, V1{base + (uint32_t)g1.x, g1.y, g1.z};
-      probes(Q.t, [&](float uu, float vv) { return sample_texels(a, V0, shift, uu, vv, wrap); },
+      probes(Q.t, wrap, [&](float uu, float vv) { return sample_texels(a, V0, shift, uu, vv, wrap); },
              [&](float uu, float vv) { return sample_texels(a, V1, shift, uu, vv, wrap); });
     } else {
       const MatDev& M = a.mats[id];
       const bool wrap = M.d.wrap;
       const MipPair Q = mip_pair(P.lod + M.log2w[k], (float)(M.mips[k] - 1));
-      probes(Q.t, [&](float uu, float vv) { return sample_bilinear(mip_view(M, k, Q.m0), uu, vv, wrap); },
+      probes(Q.t, wrap, [&](float uu, float vv) { return sample_bilinear(mip_view(M, k, Q.m0), uu, vv, wrap); },
              [&](float uu, float vv) { return sample_bilinear(mip_view(M, k, Q.m1), uu, vv, wrap); });
     }
     f[3 * k + 0] = s0 * inv;
