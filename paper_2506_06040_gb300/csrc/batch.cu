@@ -34,6 +34,9 @@ namespace nbtc {
 
 constexpr int kMaxMaterials = 1024;
 constexpr int kTileK = 128;  // pixels per classification tile
+// Warpgroups of the batched decode and the frame decode, one TMEM slot each (3 or 4 of
+// two shared-memory slots were 10 to 25% behind in every plan timed).
+constexpr int kBatchW = 4;
 constexpr int kClassifyCtas = 8 * 152;  // runs of tiles of the classification: 8 CTAs on each SM
 
 enum TileKind { kTileEmpty = 0, kTileUniform = 1, kTileMixed = 2 };
@@ -362,8 +365,7 @@ struct nbtc_batch {
   uint2* ffeat = nullptr;         // per-pixel features of the frame, 24 bytes each
   int ntruns = 0;
   // tuned configuration and graphs
-  int W = 3, Wf = 3, chunk = 32, tw = 16, th = 8;  // W: decode warpgroups, Wf: render warpgroups
-  int ta = 0, taf = 0;  // A operands in TMEM (4 warpgroups x 1 slot) for the decode / the frame
+  int chunk = 32, tw = 16, th = 8;
   cudaStream_t cap = nullptr;
   cudaGraphExec_t g_decode = nullptr, g_render = nullptr;
   nbtc_batch_info info{};
@@ -408,8 +410,8 @@ static nbtc_status enqueue_decode(nbtc_context* ctx, nbtc_batch* B, cudaStream_t
   p.chunks = B->dchunks;
   p.nchunks_dev = B->dnchunks;
   p.chunk_counter = B->dcounter;
-  p.tmem_a = B->ta;
-  return launch_tc_args(ctx, p, B->nhid, kF16, B->W, B->ta ? 1 : 2, ctx->sm_count, s);
+  p.tmem_a = 1;
+  return launch_tc_args(ctx, p, B->nhid, kF16, kBatchW, 1, ctx->sm_count, s);
 }
 
 // Lighting constants of a frame: unit directions and the half vector, in double
@@ -487,8 +489,9 @@ static nbtc_status enqueue_render(nbtc_context* ctx, nbtc_batch* B, cudaStream_t
   p.tile_w = F.tw;
   p.tile_h = F.th;
   p.tiles_x = F.tiles_x;
-  p.tmem_a = B->taf;
-  return launch_tc_args(ctx, p, B->nhid, kF16, B->Wf, B->taf ? 1 : 2, ctx->sm_count, s);
+  p.mode = kModeFrame;
+  p.tmem_a = 1;
+  return launch_tc_args(ctx, p, B->nhid, kF16, kBatchW, 1, ctx->sm_count, s);
 }
 
 static nbtc_status set_tile_shape(nbtc_batch* B, int tw, int th) {
@@ -794,60 +797,44 @@ nbtc_status nbtc_batch_create(nbtc_context* ctx, const nbtc_batch_material* mats
     NBTC_TRY(set_tile_shape(B, 16, 8));
   }
   NBTC_TRY(cuda_check(cudaStreamSynchronize(s), "plan set-up"));
-  // ---- autotune: warpgroups x chunk size (decode); warpgroups x tile shape (frame)
+  // ---- autotune: chunk size (decode), tile shape (frame)
   if (flags & NBTC_BATCH_AUTOTUNE) {
-    float best = 1e30f;
-    int bw = B->W, bc = B->chunk, bta = B->ta;
-    // candidates: 3 or 4 warpgroups of two slots with shared-memory operands,
-    // or 4 warpgroups of one slot with TMEM operands (coded as W = 5 here)
     if (B->decode_tiles > 0) {
-      for (int W : {3, 4, 5})
-        for (int c : {8, 32, 128}) {
-          B->W = W == 5 ? 4 : W;
-          B->ta = W == 5;
-          NBTC_TRY(set_decode_chunk(B, c, B->cap));
-          const float ms = time_ms([&] { return enqueue_decode(ctx, B, B->cap); }, B->cap, 3, st);
-          if (st) {
-            free_plan(B);
-            return st;
-          }
-          if (ms < best) {
-            best = ms;
-            bw = B->W;
-            bta = B->ta;
-            bc = c;
-          }
+      float best = 1e30f;
+      int bc = B->chunk;
+      for (int c : {8, 32, 128}) {
+        NBTC_TRY(set_decode_chunk(B, c, B->cap));
+        const float ms = time_ms([&] { return enqueue_decode(ctx, B, B->cap); }, B->cap, 3, st);
+        if (st) {
+          free_plan(B);
+          return st;
         }
-      B->W = bw;
-      B->ta = bta;
+        if (ms < best) {
+          best = ms;
+          bc = c;
+        }
+      }
       NBTC_TRY(set_decode_chunk(B, bc, B->cap));
       B->info.tuned_decode_ms = best;
     }
     if (B->has_frame) {
       float bestf = 1e30f;
-      int fw = B->Wf, fta = B->taf, ftw = 16, fth = 8;
+      int ftw = 16, fth = 8;
       const int shapes[4][2] = {{16, 8}, {32, 4}, {8, 16}, {128, 1}};
-      for (int W : {3, 4, 5})
-        for (auto& sh : shapes) {
-          if (set_tile_shape(B, sh[0], sh[1])) continue;
-          B->Wf = W == 5 ? 4 : W;
-          B->taf = W == 5;
-          const float ms = time_ms([&] { return enqueue_render(ctx, B, B->cap); }, B->cap, 3, st);
-          if (st) {
-            free_plan(B);
-            return st;
-          }
-          if (ms < bestf) {
-            bestf = ms;
-            fw = B->Wf;
-            fta = B->taf;
-            ftw = sh[0];
-            fth = sh[1];
-          }
+      for (auto& sh : shapes) {
+        if (set_tile_shape(B, sh[0], sh[1])) continue;
+        const float ms = time_ms([&] { return enqueue_render(ctx, B, B->cap); }, B->cap, 3, st);
+        if (st) {
+          free_plan(B);
+          return st;
         }
+        if (ms < bestf) {
+          bestf = ms;
+          ftw = sh[0];
+          fth = sh[1];
+        }
+      }
       NBTC_TRY(set_tile_shape(B, ftw, fth));
-      B->Wf = fw;
-      B->taf = fta;
       B->info.tuned_render_ms = bestf;
     }
   }
@@ -855,10 +842,8 @@ nbtc_status nbtc_batch_create(nbtc_context* ctx, const nbtc_batch_material* mats
   if (B->decode_tiles > 0) NBTC_TRY(capture(ctx, B, false, &B->g_decode));
   if (B->has_frame) NBTC_TRY(capture(ctx, B, true, &B->g_render));
 #undef NBTC_TRY
-  B->info.warpgroups = B->W;
-  B->info.render_warpgroups = B->Wf;
-  B->info.decode_tmem_operands = B->ta;
-  B->info.render_tmem_operands = B->taf;
+  B->info.warpgroups = B->info.render_warpgroups = kBatchW;
+  B->info.decode_tmem_operands = B->info.render_tmem_operands = 1;
   B->info.chunk_tiles = B->chunk;
   B->info.tile_w = B->tw;
   B->info.tile_h = B->th;

@@ -255,7 +255,7 @@ nbtc_status launch_tc_args(nbtc_context* ctx, const TcArgs& p, int nhid, int for
   (void)ctx;
   if (nhid < 1 || nhid > 3) return fail(NBTC_ERR_UNSUPPORTED, "tensor-core decode takes 1..3 hidden layers");
   using Fn = nbtc_status (*)(const TcArgs&, int, int, int, cudaStream_t);
-  if (p.mode == kModeBatch) {
+  if (p.mode == kModeBatch || p.mode == kModeFrame) {
     if (form != kF16) return fail(NBTC_ERR_UNSUPPORTED, "batched decode runs the FP16 form");
     static const Fn batch[3] = {launch_tc_h1_f16_batch, launch_tc_h2_f16_batch, launch_tc_h3_f16_batch};
     return batch[nhid - 1](p, W, slots, grid, s);

@@ -93,7 +93,7 @@ struct WorkChunk {
   int pad;
 };
 
-enum TcMode { kModeSingle = 0, kModeBatch = 1, kModeInPlace = 2 };
+enum TcMode { kModeSingle = 0, kModeBatch = 1, kModeInPlace = 2, kModeFrame = 3 };
 
 struct TcArgs {
   DecodeArgs d;

@@ -183,8 +183,8 @@ __host__ __device__ inline TcSmem tc_smem(const TcLayout& L, int W, int NSL, boo
 // wait it stops waiting but still makes every arrival -- so both barrier kinds
 // always complete and the kernel always terminates.
 // MODE kModeSingle: one material whose views are kernel parameters; kModeInPlace:
-// the same with the MLP laid out by each CTA (FP32 decodes); kModeBatch:
-// chunks of many materials (and frame tiles) whose views live in shared memory.
+// the same with the MLP laid out by each CTA (FP32 decodes); kModeBatch: chunks of
+// many materials' grids, kModeFrame: of frame tiles, whose views live in shared memory.
 template <int NHID, int FORM, int W, int MODE, int NSL, bool TA = false>
 __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
   constexpr TcLayout L{NHID, FORM};
@@ -264,6 +264,8 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
   }
   // FP32 decodes bring no packed image: each CTA lays the MLP out in its shared memory
   constexpr bool kInPlace = MODE == kModeInPlace;
+  constexpr bool kChunks = MODE == kModeBatch || MODE == kModeFrame;  // work taken from a chunk list
+  constexpr bool frame_chunk = MODE == kModeFrame;
   static_assert(!kInPlace || (FORM == kF32Split && TA), "FP32 decodes: the FP32-accurate form on TMEM operands");
   bool failed = false;
   uint32_t wph = 0;  // phase of the weight barrier
@@ -273,7 +275,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
   bool first_chunk = true;
   // batch: thread 0 takes a chunk's number while the chunk before it runs
   int next_c = 0, nchunks = 0;
-  if (MODE == kModeBatch && tid == 0) {
+  if (kChunks && tid == 0) {
     nchunks = *p.nchunks_dev;
     next_c = atomicAdd(p.chunk_counter, 1);
   }
@@ -282,7 +284,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
     // ---- take the next chunk (thread 0), load its material's MLP if it changed
     if (tid == 0) {
       int valid = 0, reload = 0;
-      if (MODE != kModeBatch) {
+      if (!kChunks) {
         if (first_chunk) {
           const int64_t b = (int64_t)blockIdx.x * p.per_cta;
           const int64_t e = b + p.per_cta < p.tiles ? b + p.per_cta : p.tiles;
@@ -318,7 +320,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
     first_chunk = false;
     if (!work.valid) break;
     if (work.reload) {
-      if (MODE == kModeBatch) {  // the material's view, by all threads (published by the barrier below)
+      if (kChunks) {  // the material's view, by all threads (published by the barrier below)
         const uint32_t* from = reinterpret_cast<const uint32_t*>(p.mats + work.c.mat);
         uint32_t* to = reinterpret_cast<uint32_t*>(&work.m);
         for (int i = tid; i < (int)(sizeof(MatDev) / 4); i += W * kTile + 32 * W) to[i] = __ldg(from + i);
@@ -351,8 +353,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
       }
     }
     failed = __syncthreads_or(failed);
-    const bool grid_chunk = work.c.kind == kChunkGrid;
-    const bool footprint = MODE != kModeBatch ? p.footprint != 0 : grid_chunk;
+    const bool footprint = kChunks ? MODE == kModeBatch : p.footprint != 0;
     const int64_t range_end = work.c.count;   // tiles are numbered 0 .. count-1 inside the chunk
 
     // Schedule.  Warpgroup g decodes the contiguous tile range [g_begin, g_end)
@@ -531,8 +532,8 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
       const uint32_t stage_s = sbase + S.stage + warp * stage_bytes(FORM);
       const float* bias = reinterpret_cast<const float*>(smem + L.off_bias());
       const float* alpha = reinterpret_cast<const float*>(smem + L.off_alpha());
-      const DecodeArgs& D = MODE != kModeBatch ? p.d : work.m.d;
-      const FastDiv& hdiv = MODE != kModeBatch ? p.hdiv : work.m.hdiv;
+      const DecodeArgs& D = kChunks ? work.m.d : p.d;
+      const FastDiv& hdiv = kChunks ? work.m.hdiv : p.hdiv;
       const int nout = work.m.nout;
       const bool whole_rows = p.whole_rows != 0;
       const int64_t g_begin = min((int64_t)wg * per_wg, range_end);
@@ -594,13 +595,12 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
       // frame chunks: this thread's pixel of each slot's tile and of the slot's next
       // tile, whose list lookups are issued a tile ahead
       int cur_px[kSlots] = {}, next_px[kSlots] = {};
-      const bool frame_chunk = MODE == kModeBatch && !grid_chunk;
       auto pixel_of = [&](int64_t T) { return T < g_end ? (int)frame_pixel(p, work.c, T, gt) : -1; };
 
       // the packed A0 row of this thread's row of tile T: from the features of its
       // texel, or (frame chunks, FP16 only) the row the feature pass left for its pixel px
       auto tile_row = [&](int64_t T, int px, uint32_t (&av)[16]) {
-        if (MODE != kModeBatch || grid_chunk) {
+        if constexpr (!frame_chunk) {
           float f[12];
           tile_features(T, f);
           pack_a0(f, av);
@@ -945,7 +945,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             __syncwarp();
             put_staged<4>(dst, stage_s, off, 4u * (uint32_t)(wr.live * nout), lane);
           }
-        } else if (MODE != kModeBatch || grid_chunk) {
+        } else if constexpr (!frame_chunk) {
           const WarpRows wr = warp_rows(D, hdiv, footprint, work.c.first + T, wq);
           if (MODE == kModeBatch || whole_rows) {  // 64 nout bytes at a multiple of 16: one bulk copy
             if (lane == 0) bulk_wait_read0();
@@ -1035,6 +1035,8 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             if constexpr (!TA) failed = __any_sync(0xffffffffu, failed);  // one failure state per warp
             tc_fence_after();
             if (l < NHID) {
+              // the next tile's feature rows on their way while this tile runs
+              if (frame_chunk && l == 0 && next_px[s] >= 0) prefetch_l1(p.ffeat + 3 * (int64_t)next_px[s]);
               hidden_epilogue(s, l);
               if constexpr (TA) {
                 // the next tile's features while the output layer's MMAs run
