@@ -435,7 +435,7 @@ typedef struct {
   float tuned_decode_ms, tuned_render_ms;  /* autotuner's best times (0 = not tuned) */
   int32_t render_warpgroups;                /* tile groups per CTA of the frame decode */
   int32_t decode_tmem_operands;             /* 1: the decode's MMA A operands live in tensor memory
-                                               (one tile slot per group), 0: in shared memory (two) */
+                                               (one tile slot per group; the only form built) */
   int32_t render_tmem_operands;             /* the same for the frame decode */
 } nbtc_batch_info;
 

@@ -294,11 +294,10 @@ static nbtc_status launch_decode_form(nbtc_context* ctx, const DecodeArgs& a, co
 // Whether a decode walks its grid in column strips of 128-texel tiles, whose
 // latent columns are decoded once per pair of rows.  The last strip of a row that
 // 128 does not divide is decoded past the row's end, so the rule bounds what that
-// wastes: 2.1 M texels in whole strips take 61 us in FP16 (12-64-64-9) and 122 us in
-// split FP16 (12-64-64-64-9), sampled texel by texel (16 BC1 taps each) 188 us and
-// 272 us, so strips win up to 2.2 decoded texels per texel in the slower form and
-// the line is at 2.  It does not depend on the rows, so a band of rows is decoded
-// as the whole grid is.
+// wastes: 2.1 M texels of 12-64-64-64-9 in whole strips take 52 us in FP16 and 96 us
+// in split FP16, sampled texel by texel (16 BC1 taps each) 136 us and 187 us, so
+// strips win up to 2.6 and 1.95 decoded texels per texel and the line is at 2.  It
+// does not depend on the rows, so a band of rows is decoded as the whole grid is.
 static bool strip_grid(const DecodeArgs& a) {
   if (a.uv || a.grid_w < 1) return false;
   const int64_t padded = (int64_t)((a.grid_w + kTile - 1) / kTile) * kTile;
@@ -308,7 +307,7 @@ static bool strip_grid(const DecodeArgs& a) {
 // NBTC_FP32 (packed and host_out as nbtc_decode takes them): the FP32-accurate
 // form with the MLP laid out by each CTA; UNSUPPORTED, with nothing launched, for
 // shapes that stay with the FFMA kernels.  Taken at hidden width 64, where it is
-// as accurate as they are (f32s_pack.cuh) and 4096^2 12-64-64-9 takes 650 us
+// as accurate as they are (f32s_pack.cuh) and 4096^2 12-64-64-9 takes 596 us
 // against 4060; narrower networks are less accurate here than in FFMA.  The rule is
 // the shape alone, so bands, host outputs and uv lists give the whole grid's bits.
 nbtc_status launch_decode_fp32_tc(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, bool host_out,

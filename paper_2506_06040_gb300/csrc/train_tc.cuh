@@ -21,7 +21,8 @@
 // the latent gradients, and the tile's weight gradients are added to the running
 // sums, by the finishing warps meanwhile.  A tile took 26.8k cycles with all of it in the
 // chain, now 20.8k (shared memory, whose bandwidth MMA operands, tile stores and the
-// atomics share, is busy 70% of it); a step at 2^20 samples 612 us, now 536.
+// atomics share, is busy 70% of it); a step at 2^20 samples 612 us,
+// now 497 (the small launches around the kernel included in both).
 //
 // The weight-gradient products reduce over the tile's samples: their operands are
 // the same shared-memory tiles read MN-major (the instruction's transpose bits),
@@ -31,8 +32,8 @@
 // columns -- an accumulator chain over all of a warpgroup's samples would lose FP32
 // accuracy as it grows.  At the end the running sums are scaled, the two warpgroups
 // added (with the rounding error kept as the compensation) and written as the CTA's
-// partial sums.  The loss and db3 use per-thread Neumaier sums and a fixed-order CTA
-// reduction, as the SIMT kernel does.
+// partial sums.  The loss and db3 use compensated per-thread sums (two-sum) and a
+// fixed-order CTA reduction.
 #pragma once
 
 #include <type_traits>

@@ -119,6 +119,21 @@ def test_decode_uv_list(nb, ctx, address):
     assert max_abs(y.cpu().numpy(), ref) <= TOL_FP32
 
 
+@pytest.mark.parametrize("dims", [[12, 32, 9], [12, 64, 9]])
+@pytest.mark.parametrize("address", ["clamp", "wrap"])
+def test_shifts_past_half_a_texel(nb, ctx, dims, address):
+    """Level shifts past half a texel, several periods of a 4-texel level included:
+    taps wrap (or clamp) into the level, on uv lists and on grids."""
+    wl = synth.small_decode_workload(128, dims, seed=79, shifts=(0.75, -3.25, 9.5, -63.5), address=address)
+    mat = nb.Material.from_synth(wl.material)
+    uv = synth.random_uv(80, 3001, lo=-1.5, hi=2.5)
+    y = nb.decode(ctx, mat, uv=torch.from_numpy(uv).cuda())
+    g = nb.decode(ctx, mat, grid=(128, 40))
+    ctx.sync()
+    assert max_abs(y.cpu().numpy(), oracle.decode.decode_uv(wl.material, uv)) <= TOL_FP32
+    assert max_abs(g.cpu().numpy(), oracle.decode.decode_grid(wl.material, 128, 40)) <= TOL_FP32
+
+
 @pytest.mark.parametrize("dims,layout", [([12, 16, 9], "B"), ([12, 32, 9], "B"), ([12, 64, 9], "B"),
                                          ([12, 32, 32, 9], "B"), ([12, 64, 64, 64, 9], "B"), ([12, 16, 16, 9], "A"),
                                          ([12, 32, 32, 32, 9], "A"), ([12, 16, 16, 16, 9], "B")])
