@@ -375,3 +375,48 @@ def test_resume_from_checkpoint(nb, ctx, tmp_path):
     for k in range(4):
         assert (a.latents[k] - b.latents[k]).abs().max().item() <= 1e-6
     assert a.step_count == b.step_count == 3
+
+
+def test_steps_repeat_bit_for_bit_at_full_size(nb, ctx):
+    """A first step of 2^20 samples from one state, ten times, and a second step from
+    one state, five times: loss, MLP gradients and MLP parameters are sums in a fixed
+    order, so they are the same bits every time; a missing wait between the kernel's
+    roles would not leave them so.  Latent gradients are FP32 atomics, whose order is
+    free: a texel's n terms (about 4 on the finest level, 256 on the coarsest) summed
+    in two orders differ by about sqrt(n) 2^-24 of their size, 1e-6 at most.  (Two
+    trajectories do part by more than that: where such a last bit of a latent carries
+    a hidden unit across its kink, one sample's gradient changes by its own size.)"""
+    from paper_2506_06040_gb300.train import ContinuousModel, padded
+    wl = synth.train_workload(full=True)
+    model = ContinuousModel.from_synth(wl)
+    tgt = padded(torch.from_numpy(wl.target).cuda())
+    uvs = [torch.from_numpy(wl.uv(step)).cuda() for step in range(2)]
+    mlp = ("weights", "biases", "m_w", "v_w", "m_b", "v_b")
+    lat = ("latents", "latent_m", "latent_v")
+
+    def take():
+        return [getattr(model, n).clone() for n in mlp], [[t.clone() for t in getattr(model, n)] for n in lat]
+
+    def put(state):
+        for n, t in zip(mlp, state[0]):
+            getattr(model, n).copy_(t)
+        for n, ts in zip(lat, state[1]):
+            for to, t in zip(getattr(model, n), ts):
+                to.copy_(t)
+
+    for step, times in ((0, 10), (1, 5)):
+        start, first = take(), None
+        for _ in range(times):
+            put(start)
+            model.step_count = step
+            loss = model.train_step(ctx, uvs[step], tgt)
+            exact = [loss, model.grad_w.clone(), model.grad_b.clone(), model.weights.clone(), model.biases.clone()]
+            grads = [g.double() for g in model.latent_grads]
+            if first is None:
+                first = (exact, grads)
+                continue
+            for got, want in zip(exact, first[0]):
+                assert torch.equal(got, want), step
+            for got, want in zip(grads, first[1]):
+                assert (got - want).norm().item() <= 1e-6 * want.norm().item(), step
+    ctx.sync()
