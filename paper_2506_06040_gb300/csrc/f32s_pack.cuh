@@ -12,7 +12,9 @@
 //    2^(T_l - T_(l-1)) at most (32 or more), which keeps their lo parts out of
 //    FP16's subnormals: at unit scale a He-initialised weight's lo part is a
 //    multiple of 2^-24, an error of 1e-7 of the weight and the largest of the
-//    form.  Output channels are scaled likewise and multiplied back in FP32.
+//    form.  Output channels are scaled likewise, to a bound that FP16 does not hold
+//    (their weights do fit), and multiplied back in FP32, where the bias is added: a
+//    bias may be any share of a channel, so it is no FP16 operand.
 //  - Accumulator rounding.  The tensor core's FP32 accumulator truncates: each
 //    MMA that adds a full-size product loses part of an ulp of the sum, always
 //    toward zero.  The hi.lo products are added first, where the sum is 2^-11 of
@@ -67,7 +69,7 @@ __device__ inline void f32s_scales(const float* __restrict__ W, const float* __r
 #pragma unroll
       for (int d = 1; d < 8; d <<= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
       if (r < o && (t & 7) == 0) {
-        s += fabsf(B[boff + r]);
+        if (l < nhid) s += fabsf(B[boff + r]);  // an output's bias is added in FP32, unscaled
         s *= 1.0001f;  // FP32 rounding of the sum
         int e = 0;
         if (s < 1e30f) frexpf(s, &e);  // s < 2^e
@@ -115,23 +117,26 @@ __device__ inline void f32s_pack(unsigned char* img, const TcLayout L, const flo
         put(base + off_sw128(n, 2 * k) + part, lo);
       }
     }
-    for (int i = t; i < o; i += nt) {
+    for (int i = t; i < o && l < nhid; i += nt) {
       uint16_t h, lo;
       split(ldexpf(B[boff + i], S.a[l + 1][i]), l == 0 ? kUlp : e, h, lo);
       if (l == 0) {
         put(L.off_w1() + off_ilv(i, 24, R1), h);
         put(L.off_w1() + off_ilv(i, 2 * (16 + 12), R1), lo);
       } else {
-        const int bt = l == nhid ? L.off_bto() : L.off_bth(l - 1);
-        put(bt + off_interleave(i, 0), h);
-        put(bt + off_interleave(i, 2), lo);
+        put(L.off_bth(l - 1) + off_interleave(i, 0), h);
+        put(L.off_bth(l - 1) + off_interleave(i, 2), lo);
       }
     }
     off += in * o;
     boff += o;
   }
-  float* mul = reinterpret_cast<float*>(img + L.off_bias()) + nhid * kHid;  // output multipliers
-  for (int c = t; c < kOutPad; c += nt) mul[c] = c < nout ? ldexpf(1.f, -S.a[nhid + 1][c]) : 0.f;
+  // output biases, then (at nhid kHid) the multipliers of the accumulated products
+  float* bias = reinterpret_cast<float*>(img + L.off_bias());
+  for (int c = t; c < kOutPad; c += nt) {
+    bias[c] = c < nout ? B[nhid * hid + c] : 0.f;
+    bias[nhid * kHid + c] = c < nout ? ldexpf(1.f, -S.a[nhid + 1][c]) : 0.f;
+  }
 }
 
 }  // namespace nbtc

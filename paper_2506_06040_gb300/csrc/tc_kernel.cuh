@@ -887,15 +887,15 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           if (odd && even_n) sts16(row + 2u * (uint32_t)(nout - 1), (uint16_t)last);
         };
         if constexpr (OUT32) {
-          // back from the channels' power-of-two scales (f32s_pack.cuh)
+          // back from the channels' power-of-two scales, and the bias (f32s_pack.cuh)
 #pragma unroll
           for (int k = 0; k < kMaxOut; k += 4) {
             if (k >= nout) break;
-            const float4 m = *reinterpret_cast<const float4*>(b + k);
-            r[k] = __float_as_uint(__uint_as_float(r[k]) * m.x);
-            r[k + 1] = __float_as_uint(__uint_as_float(r[k + 1]) * m.y);
-            r[k + 2] = __float_as_uint(__uint_as_float(r[k + 2]) * m.z);
-            r[k + 3] = __float_as_uint(__uint_as_float(r[k + 3]) * m.w);
+            const float4 m = *reinterpret_cast<const float4*>(b + k), c = *reinterpret_cast<const float4*>(bias + k);
+            r[k] = __float_as_uint(fmaf(__uint_as_float(r[k]), m.x, c.x));
+            r[k + 1] = __float_as_uint(fmaf(__uint_as_float(r[k + 1]), m.y, c.y));
+            r[k + 2] = __float_as_uint(fmaf(__uint_as_float(r[k + 2]), m.z, c.z));
+            r[k + 3] = __float_as_uint(fmaf(__uint_as_float(r[k + 3]), m.w, c.w));
           }
           // FP32 output (single-material grids and uv lists).  The warp's live texels
           // x nout floats are contiguous in the output: staged and written together
