@@ -7,8 +7,9 @@
 //    ReLU neuron by a power of two and its outgoing weights by the inverse is
 //    exact, so every neuron i of layer l is scaled by 2^a with
 //    bound_i 2^a < 2^T_l, bound_i = |b_i| + sum_k |w_ik| bound_k >= its largest
-//    activation (features lie in [0, 1]).  T_l grows by layer to 15, so nothing
-//    can overflow, whatever the weights, and the scaled weights of a row sum to
+//    activation (features lie in [0, 1]).  T_l grows by layer to 15, so neither an
+//    activation nor a weight from a live neuron (whose scaled bound is 2^(T_(l-1) - 1)
+//    or more) can overflow, and the scaled weights of a row sum to
 //    2^(T_l - T_(l-1)) at most (32 or more), which keeps their lo parts out of
 //    FP16's subnormals: at unit scale a He-initialised weight's lo part is a
 //    multiple of 2^-24, an error of 1e-7 of the weight and the largest of the
@@ -36,9 +37,14 @@
 
 namespace nbtc {
 
+// Instead of an exponent: a hidden neuron whose bound is 0 (no weight from a live
+// neuron, no bias).  Its activation is exactly 0, so its outgoing weights are left
+// out: no scale fits them (a pruned neuron's may be of any size, and inf * 0 is NaN).
+constexpr short kF32sDead = -32768;
+
 struct F32sScratch {
   float bound[2][kHid];
-  short a[5][kHid];  // exponent a of every neuron: features (0), hidden layers, outputs
+  short a[5][kHid];  // exponent a of every neuron: features (0), hidden layers, outputs; kF32sDead
   int bad;           // a weight or bound that is not finite, or beyond 2^100
 };
 
@@ -75,7 +81,7 @@ __device__ inline void f32s_scales(const float* __restrict__ W, const float* __r
         if (s < 1e30f) frexpf(s, &e);  // s < 2^e
         else S.bad = 1;                // (also NaN)
         S.bound[(l + 1) & 1][r] = s;
-        S.a[l + 1][r] = (short)(s > 0.f ? f32s_target(nhid, l + 1) - e : 0);
+        S.a[l + 1][r] = s > 0.f ? (short)(f32s_target(nhid, l + 1) - e) : l == nhid ? (short)0 : kF32sDead;
       }
     }
     off += in * o;
@@ -104,6 +110,7 @@ __device__ inline void f32s_pack(unsigned char* img, const TcLayout L, const flo
     const float e = l == 0 ? e1 : eh;
     for (int i = t; i < in * o; i += nt) {
       const int n = i / in, k = i - n * in;
+      if (S.a[l + 1][n] == kF32sDead || S.a[l][k] == kF32sDead) continue;  // (the image is cleared)
       uint16_t h, lo;
       split(ldexpf(W[off + i], S.a[l + 1][n] - S.a[l][k]), e, h, lo);
       if (l == 0) {
@@ -118,6 +125,7 @@ __device__ inline void f32s_pack(unsigned char* img, const TcLayout L, const flo
       }
     }
     for (int i = t; i < o && l < nhid; i += nt) {
+      if (S.a[l + 1][i] == kF32sDead) continue;
       uint16_t h, lo;
       split(ldexpf(B[boff + i], S.a[l + 1][i]), l == 0 ? kUlp : e, h, lo);
       if (l == 0) {

@@ -64,3 +64,21 @@ def test_constant_channels(nb, ctx, dims):
     z = nb.decode(ctx, mat, nb.FP32_TC, nb.pack_mlp(ctx, mat, nb.FP32_TC), grid=(64, 4))
     ctx.sync()
     assert bool((z[:, 0] == 0.5).all()) and bool((z[:, 4] == 0.0).all())
+
+
+@pytest.mark.parametrize("dims", SHAPES)
+@pytest.mark.parametrize("layer", ["first", "last"])
+@pytest.mark.parametrize("share", ["one", "half", "all"])
+def test_pruned_neurons(nb, ctx, dims, layer, share):
+    """Hidden neurons without an incoming weight or a bias: their activation is 0,
+    whatever their outgoing weights, which are ordinary for one and beyond any
+    finite scale for the other."""
+    wl = synth.small_decode_workload(256, dims, seed=720 + len(dims) + dims[1])
+    mlp = wl.material.mlp
+    l = 0 if layer == "first" else len(dims) - 3
+    n = {"one": 1, "half": dims[1] // 2, "all": dims[1]}[share]
+    rows = np.random.default_rng(n).permutation(dims[1])[:n]
+    mlp.weights[l][rows] = 0.0
+    mlp.biases[l][rows] = 0.0
+    mlp.weights[l + 1][:, rows[0]] *= np.float32(1e20)
+    _check(nb, ctx, wl)
