@@ -978,6 +978,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             __syncwarp();
             stage_row0();
             fence_proxy_async_smem();
+            __syncwarp();  // the copies below read rows that other lanes staged
             const int first = __shfl_sync(0xffffffffu, px, (lane * p.fseg) & 31);
             if (lane < runs) {
               const uint32_t bytes = 2u * (uint32_t)(p.fseg * nout);

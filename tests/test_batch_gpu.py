@@ -139,6 +139,28 @@ def test_frame_anisotropic_filter_all_pixels(nb, ctx, max_aniso):
     plan.close()
 
 
+@pytest.mark.parametrize("size", [(1024, 512), (128, 128)])
+def test_frame_of_whole_tiles_repeats(nb, ctx, size):
+    """Frames of mostly uniform tiles, whose output rows are staged by all lanes of a
+    warp and copied by a few: every render writes the same bits over a cleared
+    output, and they are the oracle's."""
+    w, h = size
+    bw = synth.batch_workload(num_materials=2, frame_w=w, frame_h=h, smin=256, smax=512, seed=78)
+    fr = _frame_tensors(bw)
+    plan = nb.Batch(ctx, [nb.Material.from_synth(m) for m in bw.materials], None, fr, autotune=False)
+    first = None
+    for _ in range(20):
+        fr["out"].view(torch.int16).fill_(NAN16)
+        plan.render()
+        bits = fr["out"].view(torch.int16).clone()
+        first = bits if first is None else first
+        assert torch.equal(bits, first)
+    ctx.sync()
+    assert plan.info()["frame_uniform_tiles"] > 0
+    _frame_check(bw, fr["out"], np.arange(w * h))
+    plan.close()
+
+
 @pytest.mark.parametrize("aniso", [False, True])
 @pytest.mark.parametrize("address", ["wrap", "clamp"])
 @pytest.mark.parametrize("size,side", [((128, 64), 1024), ((144, 72), 256), ((512, 256), 1024)])
