@@ -27,13 +27,13 @@
 #include <string>
 #include <vector>
 
+#include "frame_slots.h"
 #include "host.h"
 #include "tc.cuh"
 
 namespace nbtc {
 
 constexpr int kMaxMaterials = 1024;
-constexpr int kTileK = 128;  // pixels per classification tile
 // Warpgroups of the batched decode and the frame decode, one TMEM slot each (3 or 4 of
 // two shared-memory slots were 10 to 25% behind in every plan timed).
 constexpr int kBatchW = 4;
@@ -174,7 +174,7 @@ __device__ __forceinline__ int block_scan(int x, int& total, int* warp_sums) {
 __device__ void frame_scan(const FrameDev& F, int* coff, int* warp_sums) {
   const int t = threadIdx.x;
   int tiles = 0;
-  for (int m = t; m < F.nmat; m += blockDim.x) tiles += F.ucount[m] + (F.pcount[m] + kTileK - 1) / kTileK;
+  for (int m = t; m < F.nmat; m += blockDim.x) tiles += F.ucount[m] + packed_tiles(F.pcount[m]);
   int all = 0;
   block_scan(tiles, all, warp_sums);
   const int chunk = max(16, (all + 4 * F.decode_ctas - 1) / (4 * F.decode_ctas));
@@ -183,7 +183,7 @@ __device__ void frame_scan(const FrameDev& F, int* coff, int* warp_sums) {
     const int m = m0 + t;
     const int U = m < F.nmat ? F.ucount[m] : 0;
     const int px = m < F.nmat ? F.pcount[m] : 0;
-    const int P = (px + kTileK - 1) / kTileK;
+    const int P = packed_tiles(px);
     const int C = (U + chunk - 1) / chunk + (P + chunk - 1) / chunk;
     int tu, tp, tc;
     const int u = su + block_scan(U, tu, warp_sums), q = sp + block_scan(P, tp, warp_sums),
@@ -192,7 +192,8 @@ __device__ void frame_scan(const FrameDev& F, int* coff, int* warp_sums) {
       F.uoff[m] = u;
       F.poff[m] = q;
       coff[m] = c;
-      for (int i = px; i < P * kTileK; ++i) F.plist[(int64_t)q * kTileK + i] = -1;  // the last packed tile's free slots
+      const int64_t end = packed_slot(q + P, 0);
+      for (int i = free_slots(px); i > 0; --i) F.plist[end - i] = -1;  // the last packed tile's free slots
     }
     su += tu;
     sp += tp;
@@ -212,7 +213,7 @@ __device__ void frame_scan(const FrameDev& F, int* coff, int* warp_sums) {
       if (coff[mid] <= c) lo = mid;
       else hi = mid - 1;
     }
-    const int m = lo, U = F.ucount[m], P = (F.pcount[m] + kTileK - 1) / kTileK;
+    const int m = lo, U = F.ucount[m], P = packed_tiles(F.pcount[m]);
     const int nu = (U + chunk - 1) / chunk;
     int i = c - coff[m];
     if (i < nu) {
@@ -230,12 +231,12 @@ __device__ void frame_scan(const FrameDev& F, int* coff, int* warp_sums) {
 // run's places were taken in pass A, so the cursors are shared-memory ones
 // (one atomic per material present in a warp).
 __global__ void __launch_bounds__(256) k_frame_bin(FrameDev F) {
-  extern __shared__ int cur[];  // [nmat] next slot in ulist, [nmat] next slot in plist
+  extern __shared__ int cur[];  // [nmat] next slot in ulist, [nmat] next place among the material's packed pixels
   int* cu = cur;
   int* cp = cur + F.nmat;
   for (int m = threadIdx.x; m < F.nmat; m += blockDim.x) {  // places of materials the run does not hold are not used
     cu[m] = F.uoff[m] + F.ubase[(size_t)blockIdx.x * F.nmat + m];
-    cp[m] = F.poff[m] * kTileK + F.pbase[(size_t)blockIdx.x * F.nmat + m];
+    cp[m] = F.pbase[(size_t)blockIdx.x * F.nmat + m];
   }
   __syncthreads();
   const int lane = threadIdx.x & 31;
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(256) k_frame_bin(FrameDev F) {
         if (id >= 0 && lane == leader) base = atomicAdd_block(cp + id, __popc(peers));
         base = __shfl_sync(0xffffffffu, base, leader);
         if (id >= 0) {
-          int64_t slot = (int64_t)base + __popc(peers & lt);
+          int64_t slot = packed_slot(F.poff[id], base + __popc(peers & lt));
           NBTC_CHECK_INDEX(slot, F.plist_cap, F.status);
           F.plist[slot] = px + i;
         }
