@@ -719,7 +719,15 @@ nbtc_status nbtc_batch_create(nbtc_context* ctx, const nbtc_batch_material* mats
       for (int k = 0; k < 4; ++k) texels += 16 * (int64_t)level_blocks(m, k);
     NBTC_TRY(cuda_check(cudaMalloc(&B->ffeat, (size_t)frame->width * frame->height * 3 * sizeof(uint2)), "frame features"));
     if (frame_texels_rule(md, texels, (int64_t)frame->width * frame->height)) {
-      NBTC_TRY(cuda_check(cudaMalloc(&B->texels, (size_t)texels * sizeof(uint32_t)), "frame texels"));
+      const cudaError_t e = cudaMalloc(&B->texels, (size_t)texels * sizeof(uint32_t));
+      if (e == cudaErrorMemoryAllocation) {  // no room for them: BC1 at the taps, which needs none
+        cudaGetLastError();
+        B->texels = nullptr;
+      } else {
+        NBTC_TRY(cuda_check(e, "frame texels"));
+      }
+    }
+    if (B->texels) {
       std::vector<TexelRun> runs;
       std::vector<FrameLevel> levels((size_t)count * 4);
       int64_t at = 0;

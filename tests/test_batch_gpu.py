@@ -198,6 +198,33 @@ def test_frame_decoded_texels_and_bc1_taps(nb, ctx, size, side, address, aniso):
     plan.close()
 
 
+def test_frame_plan_without_room_for_texels(nb, ctx):
+    """A plan whose decoded texels (about 0.5 GB) do not fit the device's free memory
+    reads BC1 at the taps instead of failing; the frame is the oracle's."""
+    w, h = 3840, 2160
+    small = synth.batch_workload(num_materials=3, frame_w=128, frame_h=64, smin=1024, smax=1024, seed=91)
+    plan = nb.Batch(ctx, [nb.Material.from_synth(m) for m in small.materials], None, _frame_tensors(small), autotune=False)
+    plan.render()  # (the kernels of the other path are loaded)
+    plan.close()
+    bw = synth.batch_workload(num_materials=4, frame_w=w, frame_h=h, smin=16384, smax=16384, seed=92)
+    texels = sum(sum(16 * len(b) for lv in m.levels for b in lv.blocks) for m in bw.materials)
+    assert 115e6 < texels <= 16 * w * h
+    mats, fr = [nb.Material.from_synth(m) for m in bw.materials], _frame_tensors(bw)
+    ctx.sync()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    hog = torch.empty(free - (410 << 20), dtype=torch.uint8, device="cuda")  # features, lists and tables need about 270 MB
+    try:
+        plan = nb.Batch(ctx, mats, None, fr, autotune=False)
+        plan.render()
+        ctx.sync()
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    _frame_check(bw, fr["out"], np.sort(np.random.default_rng(6).integers(0, w * h, 4000)))
+    plan.close()
+
+
 def test_frame_lighting_pass(nb, ctx):
     """The fused lighting pass against the oracle's shading of the same FP16
     G-buffer values the kernel produced.  FP32 vs FP64: the GGX term is the only
