@@ -37,7 +37,7 @@ constexpr int kMaxMaterials = 1024;
 // Warpgroups of the batched decode and the frame decode, one TMEM slot each (3 or 4 of
 // two shared-memory slots were 10 to 25% behind in every plan timed).
 constexpr int kBatchW = 4;
-constexpr int kClassifyCtas = 8 * 152;  // runs of tiles of the classification: 8 CTAs on each SM
+constexpr int kClassifyPerSm = 8;  // the classification's CTAs on each SM, each with a run of tiles
 
 enum TileKind { kTileEmpty = 0, kTileUniform = 1, kTileMixed = 2 };
 
@@ -60,7 +60,8 @@ struct FrameDev {
   int* counter;  // next chunk of the decode kernel (zeroed by the scan)
   int chunk_cap;
   int decode_ctas;  // CTAs of the decode kernel
-  int ctas;         // CTAs of the classification and the binning, each with a run of tiles
+  int max_ctas;     // at most so many CTAs of the classification and the binning, each with a run of tiles
+  int ctas;         // those of the tile shape
   int per_cta;      // tiles of a run
   int ids16;        // mat_id may be read four pixels at a time
   int* stats;    // [uniform tiles, mixed tiles, packed tiles]
@@ -502,7 +503,7 @@ static nbtc_status set_tile_shape(nbtc_batch* B, int tw, int th) {
   F.th = th;
   F.tiles_x = F.w / tw;
   F.tiles = F.tiles_x * (F.h / th);
-  F.per_cta = std::max(8, (F.tiles + kClassifyCtas - 1) / kClassifyCtas);  // at least a tile per warp
+  F.per_cta = std::max(8, (F.tiles + F.max_ctas - 1) / F.max_ctas);  // at least a tile per warp
   F.ctas = (F.tiles + F.per_cta - 1) / F.per_cta;
   B->tw = tw;
   B->th = th;
@@ -773,11 +774,12 @@ nbtc_status nbtc_batch_create(nbtc_context* ctx, const nbtc_batch_material* mats
     F.h = frame->height;
     F.nmat = count;
     F.decode_ctas = ctx->sm_count;
+    F.max_ctas = kClassifyPerSm * ctx->sm_count;
     F.ids16 = aligned(frame->mat_id, 16) && frame->width % 4 == 0;
     const int pixels = frame->width * frame->height;
     const int max_tiles = pixels / kTileK + 1;
     B->plist_ints = (size_t)(pixels / kTileK + count + 1) * kTileK;
-    const size_t runs = std::min(kClassifyCtas, max_tiles / 8 + 1);
+    const size_t runs = std::min(F.max_ctas, max_tiles / 8 + 1);
     const size_t ints = (size_t)2 * count + 3 /* counts + stats */ + 2 * (size_t)count /* offsets */ +
                         2 * runs * count /* places */ + 2 * (size_t)max_tiles /* kind, mat */ + max_tiles /* ulist */ +
                         B->plist_ints + 1;
