@@ -63,11 +63,13 @@ typedef enum {
  * decode: FP16 3.2e-3 -> 9.8e-4, the FP16 output rounding; E4M3 0.37 -> 1.2e-2;
  * before the output rounding the FP16 split is within ~1e-6, which NBTC_FP32_TC
  * keeps by writing FP32, with every neuron scaled into FP16's range by a power of
- * two). */
+ * two, lo(A) lo(W) and, for layer 1, third parts added). */
 typedef enum {
   NBTC_FP32 = 0,            /* FP32 weights in, FP32 accuracy, FP32 output: FP32 FMAs
-                               (FFMA); at hidden width 64, where it is at least as
-                               accurate, NBTC_FP32_TC's arithmetic                    */
+                               (FFMA); at hidden width 64 NBTC_FP32_TC's arithmetic,
+                               whose error is 0.4 .. 0.9 of FFMA's (2-norm, measured)
+                               on networks whose rows hold many weights and up to
+                               1.4 times it, 1.5e-7, where they hold a few            */
   NBTC_FP16 = 1,            /* FP16 operands on tcgen05, FP32 accumulate, FP16 output */
   NBTC_FP8_E4M3 = 2,        /* E4M3 operands on tcgen05 with per-layer power-of-two
                                scales, FP32 accumulate, FP16 output                   */

@@ -194,8 +194,16 @@ __device__ __forceinline__ float3 bc1_texel_f(const Bc1Block& b, int tx, int ty)
   return make_float3(ch(num & 0x3FFu), ch((num >> 10) & 0x3FFu), ch(num >> 20));
 }
 
-// Bilinear sample of one BC1 level at an address_uv coordinate, FP32, channels in
-// [0, 1]: the horizontal blends of both rows as packed FP32 pairs, then the vertical one.
+// What a texel byte counts: 1/255, channels in [0, 1], or (P64) 1/64, which is exact,
+// for readers that take 64/255 into their weights.
+template <bool P64>
+__device__ __forceinline__ constexpr float texel_unit() {
+  return P64 ? 1.0f / 64.0f : 1.0f / 255.0f;
+}
+
+// Bilinear sample of one BC1 level at an address_uv coordinate, FP32: the horizontal
+// blends of both rows as packed FP32 pairs, then the vertical one.
+template <bool P64 = false>
 __device__ __forceinline__ float3 sample_bilinear(const LevelView& L, float u, float v, bool wrap) {
   int x0, x1, y0, y1;
   float fx, fy;
@@ -205,7 +213,7 @@ __device__ __forceinline__ float3 sample_bilinear(const LevelView& L, float u, f
   const uint64_t b01 = __ldg(L.blocks + block_index(L, x0 >> 2, y1 >> 2)), b11 = __ldg(L.blocks + block_index(L, x1 >> 2, y1 >> 2));
   const float3 t00 = bc1_texel_f(bc1_block(b00), x0 & 3, y0 & 3), t10 = bc1_texel_f(bc1_block(b10), x1 & 3, y0 & 3);
   const float3 t01 = bc1_texel_f(bc1_block(b01), x0 & 3, y1 & 3), t11 = bc1_texel_f(bc1_block(b11), x1 & 3, y1 & 3);
-  const float s = 1.0f / 255.0f;
+  const float s = texel_unit<P64>();
   auto blend = [&](float a0, float a1, float c0, float c1) {  // (top, bottom) left and right taps
     const float2 l = make_float2(a0, a1), r = make_float2(c0, c1);
     const float2 d = __fadd2_rn(r, make_float2(-l.x, -l.y));                    // exact

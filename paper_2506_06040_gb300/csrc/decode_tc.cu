@@ -306,10 +306,11 @@ static bool strip_grid(const DecodeArgs& a) {
 
 // NBTC_FP32 (packed and host_out as nbtc_decode takes them): the FP32-accurate
 // form with the MLP laid out by each CTA; UNSUPPORTED, with nothing launched, for
-// shapes that stay with the FFMA kernels.  Taken at hidden width 64, where it is
-// as accurate as they are (f32s_pack.cuh) and 4096^2 12-64-64-9 takes 596 us
-// against 4060; narrower networks are less accurate here than in FFMA.  The rule is
-// the shape alone, so bands, host outputs and uv lists give the whole grid's bits.
+// shapes that stay with the FFMA kernels.  Taken at hidden width 64, where its error
+// is below theirs on networks as they are trained (f32s_pack.cuh) and 4096^2
+// 12-64-64-9 takes 651 us against 4060; padded to 64 neurons, widths 16 and 32 have
+// less to gain.  The rule is the shape alone, so bands, host outputs and uv lists give
+// the whole grid's bits.
 nbtc_status launch_decode_fp32_tc(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, bool host_out,
                                   cudaStream_t s) {
   int nhid;

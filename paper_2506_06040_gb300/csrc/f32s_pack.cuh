@@ -5,31 +5,43 @@
 // What a split FP16 product loses against FP32, and what is done about it:
 //  - Range.  FP16 holds 2^-24 .. 65504, FP32 networks hold anything.  Scaling a
 //    ReLU neuron by a power of two and its outgoing weights by the inverse is
-//    exact, so every neuron i of layer l is scaled by 2^a with
-//    bound_i 2^a < 2^T_l, bound_i = |b_i| + sum_k |w_ik| bound_k >= its largest
-//    activation (features lie in [0, 1]).  T_l grows by layer to 15, so neither an
-//    activation nor a weight from a live neuron (whose scaled bound is 2^(T_(l-1) - 1)
-//    or more) can overflow, and the scaled weights of a row sum to
-//    2^(T_l - T_(l-1)) at most (32 or more), which keeps their lo parts out of
+//    exact, so every neuron i of layer l is scaled by 2^a with bound_i 2^a < 2^T_l,
+//    bound_i = b_i + sum_k max(w_ik, 0) bound_k >= its largest activation (features
+//    lie in [0, 1]), and no scaled weight from a live neuron and no scaled bias
+//    beyond 2^15.  So no operand overflows; T_l grows by layer to 15, so the scaled
+//    weights of a row sum to 32 and more, which keeps their lo parts out of
 //    FP16's subnormals: at unit scale a He-initialised weight's lo part is a
 //    multiple of 2^-24, an error of 1e-7 of the weight and the largest of the
 //    form.  Output channels are scaled likewise, to a bound that FP16 does not hold
 //    (their weights do fit), and multiplied back in FP32, where the bias is added: a
 //    bias may be any share of a channel, so it is no FP16 operand.
-//  - Accumulator rounding.  The tensor core's FP32 accumulator truncates: each
-//    MMA that adds a full-size product loses part of an ulp of the sum, always
-//    toward zero.  The hi.lo products are added first, where the sum is 2^-11 of
-//    its final size, then the hi.hi chunks of 16 inputs, which leave it at 1/n ..
-//    n/n of it (on average also for sums of both signs): c (n + 1) / 2 ulp for n
-//    chunks.  Half an ulp over a mantissa in [1, 2) makes c 0.35 to 0.36 of the
-//    sum; measured 0.325 (the bias left on 12-64-9, 12-64-64-9 and 12-64-64-64-9
-//    decodes is below 1e-8).  The weights are raised by that, into the lo part.
-//  - Feature scale.  The kernels multiply texel bytes by RN32(1 / 255), 5.9e-8 too
-//    large; layer 1 takes it back the same way.
+//  - Operands.  hi + lo hold 22 to 24 bits; the features and layer 1's weights, whose
+//    products are few, come in three parts (all 24), and lo.lo is not left out.
+//  - Accumulator rounding.  The tensor core's FP32 accumulator truncates: an MMA
+//    that leaves a full-size sum takes part of an ulp off it, always toward zero,
+//    and more where its products have one sign (they are cut to a common grid
+//    first).  The small products are added first, then the bias, then the hi.hi
+//    chunks of 16 inputs, which leave the sum at 1/n .. n/n of its final size (on
+//    average also for sums of both signs): (n + 1) / 2 times the loss at full size, n
+//    the row's chunks that hold a weight.  The row's weights are raised by that.
+//    kTruncUlp and kAlignUlp are what took the mean bias off dense and all-positive
+//    networks (half an ulp over mantissas in [1, 2) would be 0.35); a lone weight that is
+//    a power of two loses nothing and is not raised.
+//  - Feature scale.  Texel bytes over 255 are rounded, and by a rounded 1 / 255;
+//    the features come as bytes over 64 and 64/255 goes into layer 1's weights.
 //
-// Against FP64 over 30 networks the form is then as accurate as the FFMA kernels
-// at hidden width 64 or better (2-norm of the error 0.89 .. 0.90 of theirs,
-// largest error 0.71 .. 0.77), equal at 32 and 1.18 times at 16; before, 2.7 to 3 times.
+// 2-norm of the error against FP64, over that of FP32 FMAs on the same networks
+// (width 64, ten networks of each kind and depth 1 / 2 / 3, 640 x 400 texels):
+//   He-initialised                           0.68 / 0.75 / 0.80
+//   fitted to a target (800 Adam steps)      0.70 / 0.73 / 0.81
+//   He, biases of 0.1 .. 0.9                 0.55 / 0.64 / 0.66
+//   all weights positive                     0.43 / 0.42 / 0.43
+//   half the weights 0                       0.71 / 0.82 / 0.90
+//   nine in ten weights 0                    0.66 / 0.86 / 1.04
+//   one weight a row, 1                      0.79 / 0.79 / 0.79
+//   one weight a row, any                    0.95 / 1.17 / 1.36
+// FP32 FMAs round once per weight that is not 0, a split product once per operand: where
+// rows hold one weight or a few the split's error is the larger, 8e-8 to 1.5e-7 in all.
 #pragma once
 
 #include "sm100.cuh"
@@ -37,29 +49,41 @@
 
 namespace nbtc {
 
-// Instead of an exponent: a hidden neuron whose bound is 0 (no weight from a live
-// neuron, no bias).  Its activation is exactly 0, so its outgoing weights are left
-// out: no scale fits them (a pruned neuron's may be of any size, and inf * 0 is NaN).
+// Instead of an exponent: a hidden neuron whose bound is 0 (its activation is
+// exactly 0 for any features).  Its weights and its outgoing weights are left out:
+// no scale fits them (a pruned neuron's may be of any size, and inf * 0 is NaN).
 constexpr short kF32sDead = -32768;
 
 struct F32sScratch {
   float bound[2][kHid];
-  short a[5][kHid];  // exponent a of every neuron: features (0), hidden layers, outputs; kF32sDead
-  int bad;           // a weight or bound that is not finite, or beyond 2^100
+  short a[5][kHid];         // exponent a of every neuron: features (0), hidden layers, outputs; kF32sDead
+  float loss[5][kHid];      // mean share of a row's sum that truncation takes
+  int bad;                  // a weight or bound that is not finite, or beyond 2^100
 };
+
+// Mean loss of an MMA that leaves a full-size sum, in 2^-23 of it: of the sum's
+// truncation, and of its products' when they all have one sign.
+constexpr float kTruncUlp = 0.27f, kAlignUlp = 0.44f;
 
 // Exponent T of the bound of layer l's scaled values (0: features; nhid + 1: outputs).
 __host__ __device__ constexpr int f32s_target(int nhid, int l) {
   return l == 0 ? 0 : l > nhid ? 23 : nhid == 1 ? 11 : nhid == 2 ? (l == 1 ? 7 : 15) : 5 * l;
 }
 
-// Fills S.a and S.bad.  `t` of `nt` threads (a multiple of 32); ends with a barrier.
+// e with x < 2^e, for x >= 0.
+__device__ __forceinline__ int exponent_above(float x) {
+  int e;
+  frexpf(x, &e);
+  return e;
+}
+
+// Fills S.a, S.loss and S.bad.  `t` of `nt` threads (a multiple of 32); ends with a barrier.
 __device__ inline void f32s_scales(const float* __restrict__ W, const float* __restrict__ B, int nhid, int hid, int nout,
                                    int t, int nt, F32sScratch& S) {
   if (t == 0) S.bad = 0;
   if (t < kHid) {
     S.bound[0][t] = 1.f;
-    S.a[0][t] = 0;
+    S.a[0][t] = 2;  // features come as texel bytes over 64
   }
   __syncthreads();
   int off = 0, boff = 0;
@@ -69,19 +93,50 @@ __device__ inline void f32s_scales(const float* __restrict__ W, const float* __r
     // eight threads a row
     for (int r0 = 0; r0 < o; r0 += nt / 8) {
       const int r = r0 + t / 8;
-      float s = 0.f;
+      float sum = 0.f, sq = 0.f, pos = 0.f;  // of x = |w| bound, of x^2, of x over the positive weights
+      float top = 0.f;                       // largest weight once the inputs are scaled
+      uint32_t seen = 0;                      // bits 0..3: chunks of 16 inputs, 4: a weight that is no power of two, 8..: weights
       if (r < o)
-        for (int k = t & 7; k < in; k += 8) s = fmaf(fabsf(W[off + r * in + k]), mb[k], s);
+        for (int k = t & 7; k < in; k += 8) {
+          const float w = W[off + r * in + k], x = fabsf(w) * mb[k];
+          sum += x;  // (a weight that is not finite shows here, whatever its input)
+          if (w == 0.f || mb[k] == 0.f) continue;
+          sq = fmaf(x, x, sq);
+          pos += w > 0.f ? x : 0.f;
+          top = fmaxf(top, ldexpf(fabsf(w), -S.a[l][k]));
+          seen = (seen | 1u << (k >> 4) | ((__float_as_uint(w) & 0x7FFFFFu) || l == 0 ? 16u : 0u)) + 256u;
+        }
 #pragma unroll
-      for (int d = 1; d < 8; d <<= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+      for (int d = 1; d < 8; d <<= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, d);
+        sq += __shfl_xor_sync(0xffffffffu, sq, d);
+        pos += __shfl_xor_sync(0xffffffffu, pos, d);
+        top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
+        const uint32_t other = __shfl_xor_sync(0xffffffffu, seen, d);
+        seen = ((seen | other) & 31u) | ((seen & ~31u) + (other & ~31u));
+      }
       if (r < o && (t & 7) == 0) {
-        if (l < nhid) s += fabsf(B[boff + r]);  // an output's bias is added in FP32, unscaled
-        s *= 1.0001f;  // FP32 rounding of the sum
-        int e = 0;
-        if (s < 1e30f) frexpf(s, &e);  // s < 2^e
-        else S.bad = 1;                // (also NaN)
-        S.bound[(l + 1) & 1][r] = s;
-        S.a[l + 1][r] = s > 0.f ? (short)(f32s_target(nhid, l + 1) - e) : l == nhid ? (short)0 : kF32sDead;
+        const float b = l < nhid ? B[boff + r] : 0.f;
+        // share of the inputs that carry the row, and how far they have one sign
+        const float many = sq > 0.f ? sum * rsqrtf(sq) : 0.f;
+        const float one_sign = sum > 0.f ? fabsf(2.f * pos - sum) / sum : 0.f;
+        const float coherent = many * many / (float)in * one_sign;
+        sum += fabsf(b);
+        if (!(sum < 1e30f) || !(top < 1e30f)) S.bad = 1;  // (also NaN)
+        // the margin covers the FP32 rounding of these sums
+        const float bound = l < nhid ? fmaxf(pos + b + 1e-5f * sum, 0.f) : sum;
+        int a = 0;
+        if (bound > 0.f && sum < 1e30f) {
+          a = f32s_target(nhid, l + 1) - exponent_above(1.0001f * bound);
+          if (top > 0.f) a = min(a, 15 - exponent_above(top));
+          if (b != 0.f) a = min(a, 15 - exponent_above(fabsf(b)));
+          a = min(max(a, -120), 120);
+        }
+        S.bound[(l + 1) & 1][r] = 1.0001f * bound;
+        S.a[l + 1][r] = l < nhid && !(bound > 0.f) ? kF32sDead : (short)a;
+        const int n = l == 0 ? 1 : __popc(seen & 15u);
+        const bool lone = (seen >> 8) <= 1 && !(seen & 16u) && b == 0.f;
+        S.loss[l + 1][r] = lone ? 0.f : 0.5f * (float)(n + 1) * (kTruncUlp + kAlignUlp * coherent) * 1.1920929e-7f;
       }
     }
     off += in * o;
@@ -94,56 +149,55 @@ __device__ inline void f32s_scales(const float* __restrict__ W, const float* __r
 __device__ inline void f32s_pack(unsigned char* img, const TcLayout L, const float* __restrict__ W,
                                  const float* __restrict__ B, int hid, int nout, int t, int nt, const F32sScratch& S) {
   const int nhid = L.nhid, R1 = L.w1_row();
-  constexpr float kUlp = 0.325f * 1.1920929e-7f;  // mean truncation of a full-size sum
-  constexpr double kInv255 = (double)(1.0f / 255.0f);
-  const float e1 = kUlp + (float)(1.0 / 255.0 / kInv255 - 1.0);
-  const float eh = kUlp * 0.5f * (float)(hid / 16 + 1);
-  auto split = [](float w, float e, uint16_t& h, uint16_t& lo) {
-    const __half hh = __float2half_rn(w);
-    h = __half_as_ushort(hh);
-    lo = __half_as_ushort(__float2half_rn(fmaf(w, e, w - __half2float(hh))));
+  auto split = [](double w, uint16_t (&part)[3]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const __half h = __float2half_rn((float)w);
+      part[i] = __half_as_ushort(h);
+      w -= (double)__half2float(h);
+    }
   };
   auto put = [&](uint32_t at, uint16_t v) { *reinterpret_cast<uint16_t*>(img + at) = v; };
+  auto raise = [&](int l, int i) { return 1.0 + (double)S.loss[l][i]; };
   int off = 0, boff = 0;
   for (int l = 0; l <= nhid; ++l) {
     const int in = l == 0 ? 12 : hid, o = l == nhid ? nout : hid;
-    const float e = l == 0 ? e1 : eh;
     for (int i = t; i < in * o; i += nt) {
       const int n = i / in, k = i - n * in;
       if (S.a[l + 1][n] == kF32sDead || S.a[l][k] == kF32sDead) continue;  // (the image is cleared)
-      uint16_t h, lo;
-      split(ldexpf(W[off + i], S.a[l + 1][n] - S.a[l][k]), e, h, lo);
+      uint16_t q[3];
+      const float w = ldexpf(W[off + i], S.a[l + 1][n] - S.a[l][k]);
+      split((l == 0 ? 256.0 / 255.0 : 1.0) * raise(l + 1, n) * w, q);
       if (l == 0) {
-        put(L.off_w1() + off_ilv(n, 2 * k, R1), h);
-        put(L.off_w1() + off_ilv(n, 2 * (16 + k), R1), h);
-        put(L.off_w1() + off_ilv(n, 2 * (32 + k), R1), lo);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) put(L.off_w1() + off_ilv(n, 2 * (16 * j + k), R1), q[j]);
       } else {
         const int base = l == nhid ? L.off_wo() : L.off_wh(l - 1);
         const int part = l == nhid ? L.wo_part() : L.wh_part();
-        put(base + off_sw128(n, 2 * k), h);
-        put(base + off_sw128(n, 2 * k) + part, lo);
+        put(base + off_sw128(n, 2 * k), q[0]);
+        put(base + off_sw128(n, 2 * k) + part, q[1]);
       }
     }
     for (int i = t; i < o && l < nhid; i += nt) {
       if (S.a[l + 1][i] == kF32sDead) continue;
-      uint16_t h, lo;
-      split(ldexpf(B[boff + i], S.a[l + 1][i]), l == 0 ? kUlp : e, h, lo);
+      uint16_t q[3];
+      split(raise(l + 1, i) * ldexpf(B[boff + i], S.a[l + 1][i]), q);
       if (l == 0) {
-        put(L.off_w1() + off_ilv(i, 24, R1), h);
-        put(L.off_w1() + off_ilv(i, 2 * (16 + 12), R1), lo);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) put(L.off_w1() + off_ilv(i, 2 * (16 * j + 12), R1), q[j]);
       } else {
-        put(L.off_bth(l - 1) + off_interleave(i, 0), h);
-        put(L.off_bth(l - 1) + off_interleave(i, 2), lo);
+        put(L.off_bth(l - 1) + off_interleave(i, 0), q[0]);
+        put(L.off_bth(l - 1) + off_interleave(i, 2), q[1]);
       }
     }
     off += in * o;
     boff += o;
   }
   // output biases, then (at nhid kHid) the multipliers of the accumulated products
-  float* bias = reinterpret_cast<float*>(img + L.off_bias());
+  float* out = reinterpret_cast<float*>(img + L.off_bias());
   for (int c = t; c < kOutPad; c += nt) {
-    bias[c] = c < nout ? B[nhid * hid + c] : 0.f;
-    bias[nhid * kHid + c] = c < nout ? ldexpf(1.f, -S.a[nhid + 1][c]) : 0.f;
+    out[c] = c < nout ? B[nhid * hid + c] : 0.f;
+    out[nhid * kHid + c] = c < nout ? ldexpf(1.f, -S.a[nhid + 1][c]) : 0.f;
   }
 }
 

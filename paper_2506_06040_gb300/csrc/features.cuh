@@ -196,8 +196,8 @@ struct StripCache {
   uint32_t rel4;   // own texel: left tap's colbuf slot per level, 8 bits each
   float fx[4];     // own texel: horizontal weight per level
   uint32_t t1;     // own job: RGB8 of texel (jx, y1) -- the next pair's (jx, y0) when the key steps by one
-  float c0[3];     // own job: texel (jx, y0), RGB / 255
-  float dc[3];     // own job: texel (jx, y1) minus texel (jx, y0), RGB / 255
+  float c0[3];     // own job: texel (jx, y0), RGB in texel units
+  float dc[3];     // own job: texel (jx, y1) minus texel (jx, y0)
   float hf, ys;    // own job (warp_strip_features): the level's height and shift - 1/2
 };
 
@@ -317,11 +317,13 @@ __device__ __forceinline__ void strip_features(const DecodeArgs& a, int j, int i
 // horizontal neighbours from the lanes that hold them -- no shared memory and
 // no barrier across warps.  A footprint of more than 32 jobs (level-to-output
 // ratios above ~1/4) samples each texel on its own.
+template <bool P64 = false>
 __device__ __forceinline__ void direct_features(const DecodeArgs& a, int64_t t, float (&feat)[12]);
 
+template <bool P64>
 __device__ __forceinline__ void warp_strip_features(const DecodeArgs& a, int j, int i0w, int lane, StripCache& C,
                                                     float (&feat)[12]) {
-  const float s = 1.0f / 255.0f;
+  const float s = texel_unit<P64>();
   if (i0w != C.i0) {  // new strip: the warp's column plan, own job, own texel's source lanes
     C.i0 = i0w;
     C.key = INT_MIN + 1;
@@ -355,7 +357,7 @@ __device__ __forceinline__ void warp_strip_features(const DecodeArgs& a, int j, 
     C.rel4 = src4;
   }
   if (C.total > 32) {  // warp-uniform: a footprint wider than the warp's lanes
-    direct_features(a, (int64_t)j * a.grid_w + i0w + lane, feat);
+    direct_features<P64>(a, (int64_t)j * a.grid_w + i0w + lane, feat);
     return;
   }
   float cv0 = 0.f, cv1 = 0.f, cv2 = 0.f;
@@ -430,11 +432,12 @@ __device__ __forceinline__ LevelView mip_view(const MatDev& M, int k, int m) {
 }
 
 // Features of one texel sampled on its own (any uv).
+template <bool P64>
 __device__ __forceinline__ void direct_features(const DecodeArgs& a, int64_t t, float (&feat)[12]) {
   const float2 tuv = texel_uv(a, t), uv = address_uv(tuv.x, tuv.y, a.wrap);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const float3 c = sample_bilinear(a.lv[k], uv.x, uv.y, a.wrap);
+    const float3 c = sample_bilinear<P64>(a.lv[k], uv.x, uv.y, a.wrap);
     feat[3 * k + 0] = c.x;
     feat[3 * k + 1] = c.y;
     feat[3 * k + 2] = c.z;

@@ -299,6 +299,13 @@ __device__ __forceinline__ void split_f16x2(float a, float b, uint32_t& hi, uint
       : "r"(hi), "h"((unsigned short)0xBC00u), "f"(a), "f"(b));
   lo = cvt_f16x2(ra, rb);
 }
+// The same in three parts, hi + lo + lo2 = v where lo2 is 2^-24 or more (FP16's
+// smallest): all 24 bits of v >= 1/2.
+__device__ __forceinline__ void split3_f16x2(float a, float b, uint32_t& hi, uint32_t& lo, uint32_t& lo2) {
+  split_f16x2(a, b, hi, lo);
+  const float2 h = f16x2_to_float2(hi), l = f16x2_to_float2(lo);
+  lo2 = cvt_f16x2((a - h.x) - l.x, (b - h.y) - l.y);
+}
 // split of (relu a, relu b) without forming relu in FP32: hi = RN16(relu v) by
 // the converting ReLU; for v < 0, hi = 0 and the residual v - hi = v rounds to
 // a negative (or zero) lo, which max(lo, -hi) = max(lo, -0) zeroes; for v >= 0,

@@ -36,8 +36,9 @@ __host__ __device__ constexpr int stage_bytes(int form) { return (form == kF32Sp
 //   FP8         [W(12) 0 x 20]                                    K = 32
 //   FP16 split  [hiW(12) hib 000 | hiW(12) lob 000 | loW(12) 0000] K = 48
 //   FP8 split   [hiW(12) 0000 | hiW(12) 0000 | loW(12) 0000 | 0 x 16]  K = 64
+//   FP32-accurate [hiW(12) hib 000 | loW(12) lob 000 | lo2W(12) lo2b 000] K = 48
 // against A0 rows [x(12) 1 000] / [x(12) 0 x 20] / [hi x(12) 1 000 | lo x(12) 1 000]
-// / [hi x(12) 0000 | lo x(12) 0000].
+// / [hi x(12) 0000 | lo x(12) 0000] / [hi x(12) 1 000 | lo x(12) 0000 | lo2 x(12) 0000].
 struct TcLayout {
   int nhid;   // hidden layers (1..3)
   int form;   // TcForm
@@ -47,7 +48,7 @@ struct TcLayout {
   __host__ __device__ int esz() const { return fp8() ? 1 : 2; }
   __host__ __device__ int parts() const { return split() ? 2 : 1; }
   __host__ __device__ int w1_row() const { return f16split() ? 96 : form == kF8Split ? 64 : 32; }
-  __host__ __device__ int a0_row() const { return f16split() ? 64 : 32; }
+  __host__ __device__ int a0_row() const { return form == kF32Split ? 96 : f16split() ? 64 : 32; }
   __host__ __device__ int wh_part() const { return kHid * kHid * esz(); }                // 64 x 64
   __host__ __device__ int wh_bytes() const { return parts() * wh_part(); }
   __host__ __device__ int bth_bytes() const { return fp8() ? 0 : kHid * 16 * 2; }       // 64 x 16 bias tile

@@ -426,7 +426,16 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
                     }
                   }
                 } else if (l == 0) {
-                  if constexpr (F16S) {
+                  if constexpr (OUT32) {
+                    // A0: hi [x 1 000] in the 8 columns at ah, lo [x 0000] at al, lo2 [x 0000]
+                    // after the hi columns: every product but the smallest three
+                    mma_f16_ts(d, ah + 8, dsc(hi_w1, lo_w1), ID_HID, 0);       // lo2 x . hi W
+                    mma_f16_ts(d, ah, dsc(hi_w1, lo_w1 + 32), ID_HID, 1);      // hi x . lo2 W + lo2 b
+                    mma_f16_ts(d, al, dsc(hi_w1, lo_w1 + 16), ID_HID, 1);      // lo x . lo W
+                    mma_f16_ts(d, al, dsc(hi_w1, lo_w1), ID_HID, 1);           // lo x . hi W
+                    mma_f16_ts(d, ah, dsc(hi_w1, lo_w1 + 16), ID_HID, 1);      // hi x . lo W + lo b
+                    mma_f16_ts(d, ah, dsc(hi_w1, lo_w1), ID_HID, 1);           // hi x . hi W + hi b
+                  } else if constexpr (F16S) {
                     // A0: hi [x 1 000] in the 8 columns at ah, lo [x 1 000] at al
                     mma_f16_ts(d, al, dsc(hi_w1, lo_w1 + 16), ID_HID, 0);  // lo x . hi W + lo b
                     mma_f16_ts(d, ah, dsc(hi_w1, lo_w1 + 32), ID_HID, 1);  // hi x . lo W
@@ -442,18 +451,21 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
                   const uint32_t db = (uint32_t)(last ? L.wo_part() : L.wh_part()) >> 4;  // lo W, 16-byte units
                   // split: the small products first, while the (truncating)
                   // accumulator is small, then hi.hi (FP32-accurate 12-64-64-9: 4.8e-7
-                  // from FP64 in 2-norm with each chunk's three together, 2.2e-7 so)
+                  // from FP64 in 2-norm with each chunk's three together, 2.2e-7 so).
+                  // FP32-accurate form: the bias between them, an output's not at all
                   if constexpr (kOnesT)
                     mma_f16_ts(d, tmem_base + kOnesCol, dsc(hi_int, lo_bt), id, 0);
-                  else
+                  else if constexpr (!OUT32)
                     mma_f16(d, dsc(hi_int, lo_ones), dsc(hi_int, lo_bt), id, 0);
                   if constexpr (F16S) {
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
+                      if constexpr (OUT32) mma_f16_ts(d, al + 8 * kk, dsc(hi_w, lo_b + db + 2 * kk), id, kk > 0);
                       mma_f16_ts(d, al + 8 * kk, dsc(hi_w, lo_b + 2 * kk), id, 1);
                       mma_f16_ts(d, ah + 8 * kk, dsc(hi_w, lo_b + db + 2 * kk), id, 1);
                     }
                   }
+                  if (OUT32 && !last) mma_f16(d, dsc(hi_int, lo_ones), dsc(hi_int, lo_bt), id, 1);
 #pragma unroll
                   for (int kk = 0; kk < 4; ++kk) mma_f16_ts(d, ah + 8 * kk, dsc(hi_w, lo_b + 2 * kk), id, 1);
                 }
@@ -461,7 +473,14 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
                 // K chunks of 32 bytes (16 FP16 / 32 E4M3), 256 bytes apart in
                 // the no-swizzle layout
                 const uint32_t la = lo(slot + S.a0, 128);
-                if constexpr (F16S) {
+                if constexpr (OUT32) {
+                  mma_f16(d, dsc(hi_a0, la + 32), dsc(hi_w1, lo_w1), ID_HID, 0);           // lo2 x . hi W
+                  mma_f16(d, dsc(hi_a0, la), dsc(hi_w1, lo_w1 + 32), ID_HID, 1);           // hi x . lo2 W + lo2 b
+                  mma_f16(d, dsc(hi_a0, la + 16), dsc(hi_w1, lo_w1 + 16), ID_HID, 1);      // lo x . lo W
+                  mma_f16(d, dsc(hi_a0, la + 16), dsc(hi_w1, lo_w1), ID_HID, 1);           // lo x . hi W
+                  mma_f16(d, dsc(hi_a0, la), dsc(hi_w1, lo_w1 + 16), ID_HID, 1);           // hi x . lo W + lo b
+                  mma_f16(d, dsc(hi_a0, la), dsc(hi_w1, lo_w1), ID_HID, 1);                // hi x . hi W + hi b
+                } else if constexpr (F16S) {
                   mma_f16(d, dsc(hi_a0, la + 16), dsc(hi_w1, lo_w1 + 16), ID_HID, 0);      // lo x . hi W + lo b
                   mma_f16(d, dsc(hi_a0, la), dsc(hi_w1, lo_w1 + 32), ID_HID, 1);           // hi x . lo W
                   mma_f16(d, dsc(hi_a0, la), dsc(hi_w1, lo_w1), ID_HID, 1);                // hi x . hi W + hi b
@@ -492,14 +511,17 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
                   }
                 } else {
                   const uint32_t lo_bt = lo(sbase + (last ? L.off_bto() : L.off_bth(l - 1)), 128);
-                  mma_f16(d, dsc(hi_int, lo_ones), dsc(hi_int, lo_bt), id, 0);
+                  if constexpr (!OUT32) mma_f16(d, dsc(hi_int, lo_ones), dsc(hi_int, lo_bt), id, 0);
                   if constexpr (SPLIT) {
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
+                      if constexpr (OUT32)
+                        mma_f16(d, dsc(hi_w, lo_a + da + 2 * kk), dsc(hi_w, lo_b + db + 2 * kk), id, kk > 0);
                       mma_f16(d, dsc(hi_w, lo_a + da + 2 * kk), dsc(hi_w, lo_b + 2 * kk), id, 1);
                       mma_f16(d, dsc(hi_w, lo_a + 2 * kk), dsc(hi_w, lo_b + db + 2 * kk), id, 1);
                     }
                   }
+                  if (OUT32 && !last) mma_f16(d, dsc(hi_int, lo_ones), dsc(hi_int, lo_bt), id, 1);
 #pragma unroll
                   for (int kk = 0; kk < 4; ++kk)
                     mma_f16(d, dsc(hi_w, lo_a + 2 * kk), dsc(hi_w, lo_b + 2 * kk), id, 1);
@@ -538,12 +560,13 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
       const bool whole_rows = p.whole_rows != 0;
       const int64_t g_begin = min((int64_t)wg * per_wg, range_end);
       const int64_t g_end = min(g_begin + per_wg, range_end);
+      constexpr int kA0 = OUT32 ? 24 : 16;  // words of a tile's A0 row
       StripCache cache;
       strip_reset(cache);
       // FP32 decodes of a uv list: this thread's texel has a NaN coordinate (its
       // features are NaN; the FFMA kernels' ReLU drops that, the conversions keep it)
       bool nan_cur[kSlots] = {}, nan_next = false;
-      uint32_t next_a0[16];  // TA: the next tile's A0, computed during the output layer's MMAs
+      uint32_t next_a0[kA0];  // TA: the next tile's A0, computed during the output layer's MMAs
 
       // the 12 features of this thread's texel of tile T (full decode)
       auto tile_features = [&](int64_t T, float (&f)[12]) {
@@ -552,16 +575,16 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           // 32 texels' latent columns and shares them by shuffles
           const uint32_t t = (uint32_t)(work.c.first + T), H = (uint32_t)D.grid_h;
           const uint32_t cb = fastdiv(t, hdiv);
-          warp_strip_features(D, (int)(t - cb * H), (int)cb * kTile + 32 * wq, lane, cache, f);
+          warp_strip_features<OUT32>(D, (int)(t - cb * H), (int)cb * kTile + 32 * wq, lane, cache, f);
         } else {
           const int64_t tex = (work.c.first + T) * kTile + gt;
-          direct_features(D, tex < D.n ? tex : D.n - 1, f);
+          direct_features<OUT32>(D, tex < D.n ? tex : D.n - 1, f);
           if (kInPlace) nan_next = f[0] != f[0];
         }
       };
       // TA: a tile's A0 row as it goes into TMEM (8 columns; split FP16: hi in
-      // av[0..7], lo in av[8..15]), and its store + A-ready
-      auto pack_a0 = [&](const float (&f)[12], uint32_t (&av)[16]) {
+      // av[0..7], lo in av[8..15], FP32-accurate: lo2 in av[16..23]), and its store + A-ready
+      auto pack_a0 = [&](const float (&f)[12], uint32_t (&av)[kA0]) {
         if constexpr (FP8) {
           // A0 row of 32 E4M3: [x(12) 0 x 20], split: [hi x(12) 0000 | lo x(12) 0000]
           const float is = alpha[NHID + 1];  // 1 / input scale
@@ -580,6 +603,11 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
                       ((uint32_t)cvt_e4m3x2(f[4 * i + 2] * is, f[4 * i + 3] * is) << 16);
             }
           }
+        } else if constexpr (OUT32) {
+#pragma unroll
+          for (int i = 0; i < 6; ++i) split3_f16x2(f[2 * i], f[2 * i + 1], av[i], av[8 + i], av[16 + i]);
+          av[6] = 0x3C00u;  // k = 12: 1.0 for the bias's three parts
+          av[7] = av[14] = av[15] = av[22] = av[23] = 0u;
         } else if constexpr (F16S) {
 #pragma unroll
           for (int i = 0; i < 6; ++i) split_f16x2(f[2 * i], f[2 * i + 1], av[i], av[8 + i]);
@@ -599,7 +627,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
 
       // the packed A0 row of this thread's row of tile T: from the features of its
       // texel, or (frame chunks, FP16 only) the row the feature pass left for its pixel px
-      auto tile_row = [&](int64_t T, int px, uint32_t (&av)[16]) {
+      auto tile_row = [&](int64_t T, int px, uint32_t (&av)[kA0]) {
         if constexpr (!frame_chunk) {
           float f[12];
           tile_features(T, f);
@@ -616,11 +644,12 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
           av[7] = 0u;
         }
       };
-      auto store_a0 = [&](int s, const uint32_t (&av)[16]) {
+      auto store_a0 = [&](int s, const uint32_t (&av)[kA0]) {
         const int q = wg * kSlots + s;
         const uint32_t ta = tmem_base + a_col(q) + lane_off;  // the slot's A (hi) columns
         tmem_st8(ta, av);
         if constexpr (F16S) tmem_st8(ta + kApart, av + 8);
+        if constexpr (OUT32) tmem_st8(ta + 8, av + 16);
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -632,7 +661,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
         const int q = wg * kSlots + s;
         const uint32_t a0 = sbase + S.slots + q * S.slot + S.a0;
         if constexpr (TA || FORM == kF16) {
-          uint32_t av[16];
+          uint32_t av[kA0];
           tile_row(T, cur_px[s], av);
           if constexpr (TA) {
             if (kInPlace) nan_cur[s] = nan_next;
@@ -649,7 +678,13 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
         float f[12];
         tile_features(T, f);
         if (kInPlace) nan_cur[s] = nan_next;
-        if constexpr (F16S) {
+        if constexpr (OUT32) {
+          uint32_t av[kA0];
+          pack_a0(f, av);
+#pragma unroll
+          for (int i = 0; i < 6; ++i)
+            sts128(a0 + off_ilv(gt, 16 * i, L.a0_row()), av[4 * i], av[4 * i + 1], av[4 * i + 2], av[4 * i + 3]);
+        } else if constexpr (F16S) {
           uint32_t h[6], r[6];
 #pragma unroll
           for (int i = 0; i < 6; ++i) split_f16x2(f[2 * i], f[2 * i + 1], h[i], r[i]);
@@ -736,8 +771,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
             if constexpr (F16S) {
               uint32_t lw[16];
 #pragma unroll
-              for (int j = 0; j < 16; ++j)
-                split_relu_f16x2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]), h[j], lw[j]);
+              for (int j = 0; j < 16; ++j) split_relu_f16x2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]), h[j], lw[j]);
               tmem_st16(aaddr + kApart + 16 * part, lw);
             } else {
 #pragma unroll
@@ -781,8 +815,7 @@ __global__ void __launch_bounds__(W * 128 + 32 * W, 1) k_decode_tc(TcArgs p) {
               const int j = 8 * c;
               uint32_t h[4], lw[4];
 #pragma unroll
-              for (int e = 0; e < 4; ++e)
-                split_relu_f16x2(__uint_as_float(r[j + 2 * e]), __uint_as_float(r[j + 2 * e + 1]), h[e], lw[e]);
+              for (int e = 0; e < 4; ++e) split_relu_f16x2(__uint_as_float(r[j + 2 * e]), __uint_as_float(r[j + 2 * e + 1]), h[e], lw[e]);
               const uint32_t o = off_sw128(gt, 16 * (part * (kPc / 8) + c));
               sts128(ah + o, h[0], h[1], h[2], h[3]);
               sts128(ah + S.ah_lo + o, lw[0], lw[1], lw[2], lw[3]);
