@@ -156,8 +156,8 @@ __device__ __forceinline__ void axis_taps(float u, int n, float shift, bool wrap
 // with F = 2^23 + num (the field under the exponent of 2^23),
 //   four colours   num = a0 e0 + a1 e1 + 1 <= 766:       RN(F / 3 + 9786709) = 2^23 + 2^22 + num div 3
 //   three colours  num = 2 (a0 e0 + a1 e1) + 1 <= 1021:  RN(F / 4 + 10485760) = 2^23 + 2^22 + (num + 1) div 4
-// (the second is (a0 e0 + a1 e1 + 1) div 2; both checked for every numerator on the
-// host against the integer form).  ~45 instructions a tap with its share of the
+// (the second is (a0 e0 + a1 e1 + 1) div 2; both tested for every numerator on the
+// host).  ~45 instructions a tap with its share of the
 // block, where the integer decode and conversion of bc1_texel took ~65.
 struct Bc1Block {
   uint32_t e0, e1;  // endpoints: r | g << 10 | b << 20
