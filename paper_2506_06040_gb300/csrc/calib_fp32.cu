@@ -1,5 +1,5 @@
-// FP8 calibration: the FP32 decode kernel recording each layer's input absmax
-// (instantiations of fp32_kernel.cuh).
+// FP8 calibration: largest magnitude of every layer's inputs (instantiations of
+// fp32_kernel.cuh).
 #include "fp32_kernel.cuh"
 
 namespace nbtc {
@@ -8,7 +8,7 @@ nbtc_status launch_calibrate_fp32(nbtc_context* ctx, const DecodeArgs& a, const 
                                   float* absmax, cudaStream_t s) {
   nbtc_status st = cuda_check(cudaMemsetAsync(absmax, 0, sizeof(float) * mlp->num_layers, s), "memset absmax");
   if (st) return st;
-  return dispatch<true>(ctx, a, mlp, step, absmax, s);
+  return dispatch(ctx, a, mlp, step, absmax, s);
 }
 
 }  // namespace nbtc

@@ -302,9 +302,10 @@ nbtc_status nbtc_fp8_calibrate(nbtc_context* ctx, const nbtc_latents* lat, const
   return launch_calibrate_fp32(ctx, a, mlp, step, act_absmax_dev, (cudaStream_t)stream);
 }
 
-// Where a decode may write: device (or managed) memory, or -- FP32 decodes,
-// whose kernels store with plain global stores -- pinned host memory, which the
-// kernel writes directly over the host link (its device address replaces out).
+// Where a decode may write: device (or managed) memory, or -- NBTC_FP32, whose
+// kernels then store with plain global stores instead of bulk copies -- pinned host
+// memory, which the kernel writes directly over the host link (its device address
+// replaces out).
 static nbtc_status resolve_out(int32_t precision, DecodeArgs& a, bool& host_out) {
   host_out = false;
   cudaPointerAttributes pa;
@@ -322,7 +323,7 @@ static nbtc_status resolve_out(int32_t precision, DecodeArgs& a, bool& host_out)
   if (pa.type == cudaMemoryTypeHost && pa.devicePointer) {
     if (precision != NBTC_FP32)
       return fail(NBTC_ERR_UNSUPPORTED,
-                  "pinned host output is for the FP32 SIMT decode; tensor-core forms decode into device memory");
+                  "pinned host output is for NBTC_FP32; the other forms decode into device memory");
     a.out = pa.devicePointer;
     host_out = true;
     if (!aligned(a.out, 16)) return fail(NBTC_ERR_INVALID_ARG, "out not 16-byte aligned");

@@ -9,7 +9,10 @@
 // once -- into shared memory; each texel then blends its two neighbouring
 // columns horizontally.  This is the bilinear filter of Sec. 3.1 evaluated in
 // separable order, with every BC1 block decoded once per tile instead of once
-// per tap.  Direct mode (uv lists, ragged grids) samples each texel on its own.
+// per tap.  The tensor-core kernels take it a warp at a time with a column cache over
+// rows, the last strip past the row's end (see strip_grid in decode_tc.cu).  Direct
+// mode (uv lists, grids too narrow for that, rows that 256 does not divide in the
+// FFMA kernel, footprints wider than the group) samples each texel on its own.
 #pragma once
 
 #include <climits>
@@ -177,135 +180,30 @@ __device__ __forceinline__ void footprint_features(const DecodeArgs& a, int64_t 
   blend_columns<NT>(a, P, tid, colbuf, feat);
 }
 
-// ---- row-footprint feature stage with a per-thread column cache, for a group
-// of NT threads that decodes vertically consecutive tiles of one column strip
-// (the same first column i0, output rows j, j+1, ...).  Across such tiles the
-// column plan, each thread's column job and each texel's horizontal taps stay
+// ---- column cache of a warp that decodes vertically consecutive tiles of one column
+// strip (the same first column i0, output rows j, j+1, ...).  Across such tiles the
+// column plan, each lane's column job and each texel's horizontal taps stay
 // fixed, and a latent column's two vertical taps (rows floor(ty), floor(ty)+1)
 // change only when ty crosses a texel boundary: every 4th output row for a
-// latent at 1/4 of the output side, every 32nd at 1/32.  So each thread keeps
-// its job's two decoded texels (as floats scaled to [0, 1]) and reloads and
-// decodes the BC1 blocks only when floor(ty) changes; per tile it only redoes
-// the vertical blend of its column and the horizontal blend of its texel.
+// latent at 1/4 of the output side, every 32nd at 1/32.  So each lane keeps
+// its job's two decoded texels (as floats) and reloads and decodes the BC1 blocks
+// only when floor(ty) changes; per tile it only redoes the vertical blend of its
+// column and the horizontal blend of its texel.
 struct StripCache {
   int i0;          // first output column of the cached strip (-1: none)
   int total;       // column jobs of the strip
-  int job;         // own job: level | colbuf slot << 2 (-1: none)
+  int job;         // own job: level | column of the level << 2 (-1: none)
   int jx;          // own job: latent column (wrapped or clamped)
   int key;         // floor(ty) of the decoded pair (INT_MIN + 1: none)
-  uint32_t rel4;   // own texel: left tap's colbuf slot per level, 8 bits each
+  uint32_t rel4;   // own texel: lane that holds its left tap, per level, 8 bits each
   float fx[4];     // own texel: horizontal weight per level
   uint32_t t1;     // own job: RGB8 of texel (jx, y1) -- the next pair's (jx, y0) when the key steps by one
   float c0[3];     // own job: texel (jx, y0), RGB in texel units
   float dc[3];     // own job: texel (jx, y1) minus texel (jx, y0)
-  float hf, ys;    // own job (warp_strip_features): the level's height and shift - 1/2
+  float hf, ys;    // own job: the level's height and shift - 1/2
 };
 
 __device__ __forceinline__ void strip_reset(StripCache& C) { C.i0 = -1; }
-
-// Features of texel i0 + tid of output row j; (j, i0) is a tile of NT texels
-// in one row (i0 + NT <= grid_w).
-template <int NT>
-__device__ __forceinline__ void strip_features(const DecodeArgs& a, int j, int i0, int tid, uint32_t colbuf,
-                                               int bar_id, StripCache& C, float (&feat)[12]) {
-  const float s = 1.0f / 255.0f;
-  if (i0 != C.i0) {  // new strip: column plan, own job, own texel's taps
-    C.i0 = i0;
-    C.key = INT_MIN + 1;  // no pair decoded (and key == C.key + 1 cannot hold)
-    const float u0 = grid_coord((float)i0, a.cw);
-    const float u1 = grid_coord((float)(i0 + NT - 1), a.cw);
-    const float u = grid_coord((float)(i0 + tid), a.cw);
-    int total = 0, job = -1, jx = 0;
-    uint32_t rel4 = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const LevelView& L = a.lv[k];
-      const int b0 = (int)floorf(texel_coord(u0, L.w, L.shift));
-      const int b1 = (int)floorf(texel_coord(u1, L.w, L.shift));
-      const int span = min(b1 - b0 + 2, kColCap);
-      if (tid >= total && tid < total + span) {
-        job = k | (tid - total) << 2;
-        jx = wrap_or_clamp(b0 + tid - total, L.w, a.wrap);
-      }
-      total += span;
-      const float tx = texel_coord(u, L.w, L.shift);
-      const float ftx = floorf(tx);
-      C.fx[k] = tx - ftx;
-      // floor is monotone in u, so the slot lies in [0, span - 2]; the clamp only guards the buffer
-      rel4 |= (uint32_t)min(max((int)ftx - b0, 0), span - 2) << (8 * k);
-    }
-    C.total = total;
-    C.job = job;
-    C.jx = jx;
-    C.rel4 = rel4;
-  }
-  if (C.job >= 0) {
-    const int k = C.job & 3;
-    const LevelView& L = a.lv[k];
-    const float ty = texel_coord(grid_coord((float)(j + a.row0), a.ch), L.h, L.shift);
-    const float fty = floorf(ty);
-    const float fy = ty - fty;
-    const int key = (int)fty;
-    if (key != C.key) {
-      // moving down one latent row, the new pair's upper texel is the old pair's
-      // lower one: decode only the new lower texel
-      uint32_t t0;
-      if (key == C.key + 1) {
-        t0 = C.t1;
-      } else {
-        const int y0 = wrap_or_clamp(key, L.h, a.wrap);
-        t0 = bc1_texel(__ldg(L.blocks + block_index(L, C.jx >> 2, y0 >> 2)), C.jx & 3, y0 & 3);
-      }
-      const int y1 = wrap_or_clamp(key + 1, L.h, a.wrap);
-      const uint32_t t1 = bc1_texel(__ldg(L.blocks + block_index(L, C.jx >> 2, y1 >> 2)), C.jx & 3, y1 & 3);
-      C.key = key;
-      C.t1 = t1;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float v0 = (float)((t0 >> (8 * c)) & 255u), v1 = (float)((t1 >> (8 * c)) & 255u);
-        C.c0[c] = s * v0;
-        C.dc[c] = s * (v1 - v0);
-      }
-    }
-    sm100::sts128f(colbuf + 16u * (uint32_t)(k * kColCap + (C.job >> 2)), fmaf(fy, C.dc[0], C.c0[0]),
-                   fmaf(fy, C.dc[1], C.c0[1]), fmaf(fy, C.dc[2], C.c0[2]), 0.f);
-    // the next row's pair changes here too: start pulling its blocks into L1
-    const float tyn = texel_coord(grid_coord((float)(j + a.row0 + 1), a.ch), L.h, L.shift);
-    const int keyn = (int)floorf(tyn);
-    if (keyn != key && j + 1 < a.grid_h) {
-      const int y1 = wrap_or_clamp(keyn + 1, L.h, a.wrap);
-      sm100::prefetch_l1(L.blocks + block_index(L, C.jx >> 2, y1 >> 2));
-    }
-  }
-  if (C.total > NT) {
-    // a strip wider than NT columns over all levels: the jobs past the first
-    // per thread are decoded afresh for every tile (only unusual level-to-output
-    // ratios get here; the 1/4..1/32 pyramid needs 68 columns per 128 texels)
-    const TilePlan P = plan_tile<NT>(a, (int64_t)j * a.grid_w + i0);
-    for (int job = tid + NT; job < P.total; job += NT) {
-      const ColumnJob J = column_job(a, P, job);
-      const BlockPair B = load_column(a, J);
-      const uint32_t t0 = bc1_texel(B.b0, J.x & 3, J.y0 & 3), t1 = bc1_texel(B.b1, J.x & 3, J.y1 & 3);
-      float c[3];
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        const float v0 = (float)((t0 >> (8 * ch)) & 255u), v1 = (float)((t1 >> (8 * ch)) & 255u);
-        c[ch] = fmaf(J.fy, s * (v1 - v0), s * v0);
-      }
-      sm100::sts128f(colbuf + 16u * (uint32_t)(J.k * kColCap + J.rel), c[0], c[1], c[2], 0.f);
-    }
-  }
-  sm100::named_bar_sync(bar_id, NT);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const uint32_t at = colbuf + 16u * (uint32_t)(k * kColCap + ((C.rel4 >> (8 * k)) & 255));
-    const float4 A = sm100::lds128f(at);
-    const float4 B = sm100::lds128f(at + 16);
-    feat[3 * k + 0] = fmaf(C.fx[k], B.x - A.x, A.x);
-    feat[3 * k + 1] = fmaf(C.fx[k], B.y - A.y, A.y);
-    feat[3 * k + 2] = fmaf(C.fx[k], B.z - A.z, A.z);
-  }
-}
 
 // ---- row-footprint feature stage of one warp, with the latent columns shared
 // between its lanes by shuffles.  The warp's 32 consecutive texels of one

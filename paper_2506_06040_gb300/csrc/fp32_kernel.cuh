@@ -1,9 +1,7 @@
-// FP32 SIMT form of the fused decode (template; instantiated in
-// decode_fp32.cu and calib_fp32.cu).
-//
-// The paper's "software FMA" path (Sec. 5, Table 2): BC1 fetch + decode +
-// bilinear sampling of the 4 latent levels, then the MLP with true FP32 fused
-// multiply-adds.  Each thread decodes TPT texels at once; with TPT = 2 every
+// FP8 calibration: the decode of every `step`-th texel of a grid in FP32 (BC1 fetch +
+// decode + bilinear sampling of the 4 latent levels, then the MLP in fused
+// multiply-adds), of which it keeps the largest magnitude of the features and of every
+// hidden layer.  Each thread decodes TPT texels at once; with TPT = 2 every
 // multiply-add is a packed FP32x2 FMA whose weight operand (duplicated in
 // shared memory) is shared by the texel pair.
 #pragma once
@@ -22,7 +20,6 @@ struct Vec<1> {
   static __device__ __forceinline__ T relu(T x) { return fmaxf(x, 0.f); }
   static __device__ __forceinline__ T splat(float x) { return x; }
   static __device__ __forceinline__ float absmax(T x) { return fabsf(x); }
-  static __device__ __forceinline__ float lane(T x, int) { return x; }
   static __device__ __forceinline__ void set(T& x, int, float v) { x = v; }
 };
 
@@ -33,7 +30,6 @@ struct Vec<2> {
   static __device__ __forceinline__ T relu(T x) { return make_float2(fmaxf(x.x, 0.f), fmaxf(x.y, 0.f)); }
   static __device__ __forceinline__ T splat(float x) { return make_float2(x, x); }
   static __device__ __forceinline__ float absmax(T x) { return fmaxf(fabsf(x.x), fabsf(x.y)); }
-  static __device__ __forceinline__ float lane(T x, int q) { return q ? x.y : x.x; }
   static __device__ __forceinline__ void set(T& x, int q, float v) {
     if (q) x.y = v; else x.x = v;
   }
@@ -110,9 +106,9 @@ __device__ __forceinline__ void dense_relu_out(const typename VV::T* __restrict_
   }
 }
 
-template <int D, int NHID, int NOUT, int TPT, bool CALIB>
+template <int D, int NHID, int NOUT, int TPT>
 __global__ void __launch_bounds__(256, 1)
-    k_decode_fp32(DecodeArgs a, const float* __restrict__ gW, const float* __restrict__ gB,
+    k_calib_fp32(DecodeArgs a, const float* __restrict__ gW, const float* __restrict__ gB,
                   int calib_step, float* __restrict__ absmax) {
   using VV = Vec<TPT>;
   using T = typename VV::T;
@@ -134,11 +130,8 @@ __global__ void __launch_bounds__(256, 1)
     sm[Lay::w_total + e] = VV::splat(gB[e]);
   __syncthreads();
 
-  int64_t nunits = a.n, cw = 0;
-  if (CALIB) {
-    cw = (a.grid_w + calib_step - 1) / calib_step;
-    nunits = cw * ((a.grid_h + calib_step - 1) / calib_step);
-  }
+  const int64_t cw = (a.grid_w + calib_step - 1) / calib_step;
+  const int64_t nunits = cw * ((a.grid_h + calib_step - 1) / calib_step);
   float amax[NHID + 1];
 #pragma unroll
   for (int l = 0; l <= NHID; ++l) amax[l] = 0.f;
@@ -151,8 +144,7 @@ __global__ void __launch_bounds__(256, 1)
     for (int q = 0; q < TPT; ++q) {
       int64_t k = g * TPT + q;
       if (k >= nunits) k = nunits - 1;
-      if (CALIB) k = (k / cw) * calib_step * a.grid_w + (k % cw) * calib_step;
-      tex[q] = k;
+      tex[q] = (k / cw) * calib_step * a.grid_w + (k % cw) * calib_step;
     }
     T x[kNin];
 #pragma unroll
@@ -166,10 +158,8 @@ __global__ void __launch_bounds__(256, 1)
         VV::set(x[3 * k + 2], q, c.z);
       }
     }
-    if (CALIB) {
 #pragma unroll
-      for (int i = 0; i < kNin; ++i) amax[0] = fmaxf(amax[0], VV::absmax(x[i]));
-    }
+    for (int i = 0; i < kNin; ++i) amax[0] = fmaxf(amax[0], VV::absmax(x[i]));
     T out[NOUT];
     const T* W = sm;
     const T* B = sm + Lay::w_total;
@@ -180,10 +170,8 @@ __global__ void __launch_bounds__(256, 1)
     } else if constexpr (NHID == 2) {
       T h1[D];
       dense_relu<kNin, D, VV>(W + Lay::w_off(0), B + Lay::b_off(0) - Lay::w_total, x, h1);
-      if (CALIB) {
 #pragma unroll
-        for (int i = 0; i < D; ++i) amax[1] = fmaxf(amax[1], VV::absmax(h1[i]));
-      }
+      for (int i = 0; i < D; ++i) amax[1] = fmaxf(amax[1], VV::absmax(h1[i]));
       dense_relu_out<D, D, NOUT, 8, VV>(W + Lay::w_off(1), B + Lay::b_off(1) - Lay::w_total,
                                         W + Lay::w_off(2), B + Lay::b_off(2) - Lay::w_total, h1, out,
                                         amax[2]);
@@ -192,60 +180,44 @@ __global__ void __launch_bounds__(256, 1)
       T h1[D], h2[D];
       dense_relu<kNin, D, VV>(W + Lay::w_off(0), B + Lay::b_off(0) - Lay::w_total, x, h1);
       dense_relu<D, D, VV>(W + Lay::w_off(1), B + Lay::b_off(1) - Lay::w_total, h1, h2);
-      if (CALIB) {
 #pragma unroll
-        for (int i = 0; i < D; ++i) {
-          amax[1] = fmaxf(amax[1], VV::absmax(h1[i]));
-          amax[2] = fmaxf(amax[2], VV::absmax(h2[i]));
-        }
+      for (int i = 0; i < D; ++i) {
+        amax[1] = fmaxf(amax[1], VV::absmax(h1[i]));
+        amax[2] = fmaxf(amax[2], VV::absmax(h2[i]));
       }
       dense_relu_out<D, D, NOUT, 8, VV>(W + Lay::w_off(2), B + Lay::b_off(2) - Lay::w_total,
                                         W + Lay::w_off(3), B + Lay::b_off(3) - Lay::w_total, h2, out,
                                         amax[3]);
     }
-    if (!CALIB) {
-      float* o = reinterpret_cast<float*>(a.out);
-#pragma unroll
-      for (int q = 0; q < TPT; ++q) {
-        if (g * TPT + q < nunits) {
-#pragma unroll
-          for (int k = 0; k < NOUT; ++k) o[tex[q] * NOUT + k] = VV::lane(out[k], q);
-        }
-      }
-    }
   }
-  if (CALIB) {
-    // non-negative floats order like their bit patterns
+  // non-negative floats order like their bit patterns
 #pragma unroll
-    for (int l = 0; l <= NHID; ++l) {
-      float m = amax[l];
-      for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-      if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<int*>(absmax) + l, __float_as_int(m));
-    }
+  for (int l = 0; l <= NHID; ++l) {
+    float m = amax[l];
+    for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<int*>(absmax) + l, __float_as_int(m));
   }
 }
 
-template <int D, int NHID, bool CALIB>
+template <int D, int NHID>
 static nbtc_status launch_t(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, int step,
                             float* absmax, cudaStream_t s) {
   constexpr int TPT = (NHID >= 3) ? 1 : 2;
   using Lay = Fp32Layout<D, NHID, 9>;
   const size_t smem = sizeof(typename Vec<TPT>::T) * Lay::total;
-  auto kern = k_decode_fp32<D, NHID, 9, TPT, CALIB>;
+  auto kern = k_calib_fp32<D, NHID, 9, TPT>;
   nbtc_status st = cuda_check(
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "smem attribute");
   if (st) return st;
-  int64_t units = a.n;
-  if (CALIB) units = (int64_t)((a.grid_w + step - 1) / step) * ((a.grid_h + step - 1) / step);
+  const int64_t units = (int64_t)((a.grid_w + step - 1) / step) * ((a.grid_h + step - 1) / step);
   const int64_t groups = (units + TPT - 1) / TPT;
   int64_t grid = (groups + 255) / 256;
   if (grid > ctx->sm_count) grid = ctx->sm_count;
   if (grid < 1) grid = 1;
   kern<<<(int)grid, 256, smem, s>>>(a, mlp->weights, mlp->biases, step, absmax);
-  return cuda_check(cudaGetLastError(), "launch k_decode_fp32");
+  return cuda_check(cudaGetLastError(), "launch k_calib_fp32");
 }
 
-template <bool CALIB>
 static nbtc_status dispatch(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, int step,
                             float* absmax, cudaStream_t s) {
   const int L = mlp->num_layers;
@@ -255,7 +227,7 @@ static nbtc_status dispatch(nbtc_context* ctx, const DecodeArgs& a, const nbtc_m
   if (mlp->dims[0] != kNin) return fail(NBTC_ERR_UNSUPPORTED, "decode kernels take 12 input features");
   if (mlp->dims[L] != 9) return fail(NBTC_ERR_UNSUPPORTED, "FP32 decode kernels output 9 channels");
 #define NBTC_CASE(DD, HH) \
-  if (D == DD && L - 1 == HH) return launch_t<DD, HH, CALIB>(ctx, a, mlp, step, absmax, s);
+  if (D == DD && L - 1 == HH) return launch_t<DD, HH>(ctx, a, mlp, step, absmax, s);
   NBTC_CASE(16, 1) NBTC_CASE(32, 1) NBTC_CASE(64, 1)
   NBTC_CASE(32, 2) NBTC_CASE(64, 2)
   NBTC_CASE(64, 3)

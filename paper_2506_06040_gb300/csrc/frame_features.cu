@@ -5,7 +5,7 @@
 // A pixel takes two bilinear samples per level (trilinear), or that many per
 // probe of the anisotropic filter: 32 to 512 dependent gathers.  Inside the
 // tensor-core kernel, whose 16 warps a SM are set by its registers and tensor
-// memory, those gathers were latency-bound; here they run at 40 to 48 warps a SM
+// memory, those gathers were latency-bound; here they run at 36 to 40 warps a SM
 // for 24 bytes a pixel written and read back.
 #include "features.cuh"
 #include "host.h"
