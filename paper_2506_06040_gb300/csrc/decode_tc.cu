@@ -79,7 +79,11 @@ __global__ void k_pack_mlp(const float* __restrict__ W, const float* __restrict_
     __shared__ F32sScratch S;
     f32s_scales(W, B, nhid, hid, nout, threadIdx.x, blockDim.x, S);
     if (S.bad) {  // weights that are not finite (or beyond any FP16 scale): unscaled, as the values fall
-      for (int e = threadIdx.x; e < 5 * kHid; e += blockDim.x) S.a[e / kHid][e % kHid] = 0;
+      for (int e = threadIdx.x; e < 5 * kHid; e += blockDim.x) {
+        S.up[e / kHid][e % kHid] = e < kHid ? 4.f : 1.f;
+        S.down[e / kHid][e % kHid] = e < kHid ? 0.25f : 1.f;
+        S.loss[e / kHid][e % kHid] = 0.f;
+      }
       __syncthreads();
     }
     f32s_pack(out, L, W, B, hid, nout, threadIdx.x, blockDim.x, S);
@@ -308,7 +312,7 @@ static bool strip_grid(const DecodeArgs& a) {
 // form with the MLP laid out by each CTA; UNSUPPORTED, with nothing launched, for
 // shapes that stay with the FFMA kernels.  Taken at hidden width 64, where its error
 // is below theirs on networks as they are trained (f32s_pack.cuh) and 4096^2
-// 12-64-64-9 takes 651 us against 4060; padded to 64 neurons, widths 16 and 32 have
+// 12-64-64-9 takes 643 us against 4060; padded to 64 neurons, widths 16 and 32 have
 // less to gain.  The rule is the shape alone, so bands, host outputs and uv lists give
 // the whole grid's bits.
 nbtc_status launch_decode_fp32_tc(nbtc_context* ctx, const DecodeArgs& a, const nbtc_mlp* mlp, bool host_out,

@@ -49,16 +49,15 @@
 
 namespace nbtc {
 
-// Instead of an exponent: a hidden neuron whose bound is 0 (its activation is
-// exactly 0 for any features).  Its weights and its outgoing weights are left out:
-// no scale fits them (a pruned neuron's may be of any size, and inf * 0 is NaN).
-constexpr short kF32sDead = -32768;
-
 struct F32sScratch {
   float bound[2][kHid];
-  short a[5][kHid];         // exponent a of every neuron: features (0), hidden layers, outputs; kF32sDead
-  float loss[5][kHid];      // mean share of a row's sum that truncation takes
-  int bad;                  // a weight or bound that is not finite, or beyond 2^100
+  // 2^a of every neuron's scale and 2^-a: features (0), hidden layers, outputs.  Both 0
+  // for a hidden neuron whose bound is 0 (its activation is exactly 0 for any
+  // features): that leaves out its weights and its outgoing weights, for which there is
+  // no scale (a pruned neuron's may be of any size, and inf * 0 is NaN).
+  float up[5][kHid], down[5][kHid];
+  float loss[5][kHid];  // mean share of a row's sum that truncation takes
+  int bad;              // a weight or bound that is not finite, or beyond 2^100
 };
 
 // Mean loss of an MMA that leaves a full-size sum, in 2^-23 of it: of the sum's
@@ -70,22 +69,28 @@ __host__ __device__ constexpr int f32s_target(int nhid, int l) {
   return l == 0 ? 0 : l > nhid ? 23 : nhid == 1 ? 11 : nhid == 2 ? (l == 1 ? 7 : 15) : 5 * l;
 }
 
-// e with x < 2^e, for x >= 0.
-__device__ __forceinline__ int exponent_above(float x) {
-  int e;
-  frexpf(x, &e);
-  return e;
-}
+// e with x < 2^e, for finite x >= 0 (subnormal ones count as 2^-127).
+__device__ __forceinline__ int exponent_above(float x) { return (int)(__float_as_uint(x) >> 23) - 126; }
 
-// Fills S.a, S.loss and S.bad.  `t` of `nt` threads (a multiple of 32); ends with a barrier.
-__device__ inline void f32s_scales(const float* __restrict__ W, const float* __restrict__ B, int nhid, int hid, int nout,
-                                   int t, int nt, F32sScratch& S) {
+// 2^a, |a| <= 126.
+__device__ __forceinline__ float pow2f(int a) { return __int_as_float((a + 127) << 23); }
+
+// Fills S (in shared memory) but for the bounds.  `t` of `nt` threads (a multiple of
+// 32); ends with a barrier.  Out of line, as f32s_pack: inlined they cost the decode
+// kernel's main loop registers (4096^2 12-64-64-9: 671 us, 643 so).
+static __device__ __noinline__ void f32s_scales(const float* __restrict__ W, const float* __restrict__ B, int nhid,
+                                                int hid, int nout, int t, int nt, F32sScratch& S) {
+  // every layer waits for the one before: all its weights on their way first
+  for (int i = 32 * t; i < 12 * hid + (nhid - 1) * hid * hid + hid * nout; i += 32 * nt) sm100::prefetch_l1(W + i);
+  if (32 * t < nhid * hid + nout) sm100::prefetch_l1(B + 32 * t);
   if (t == 0) S.bad = 0;
   if (t < kHid) {
     S.bound[0][t] = 1.f;
-    S.a[0][t] = 2;  // features come as texel bytes over 64
+    S.up[0][t] = 4.f;  // features come as texel bytes over 64
+    S.down[0][t] = 0.25f;
   }
   __syncthreads();
+  const float inv_hid = 1.f / (float)hid;
   int off = 0, boff = 0;
   for (int l = 0; l <= nhid; ++l) {
     const int in = l == 0 ? 12 : hid, o = l == nhid ? nout : hid;
@@ -95,17 +100,26 @@ __device__ inline void f32s_scales(const float* __restrict__ W, const float* __r
       const int r = r0 + t / 8;
       float sum = 0.f, sq = 0.f, pos = 0.f;  // of x = |w| bound, of x^2, of x over the positive weights
       float top = 0.f;                       // largest weight once the inputs are scaled
-      uint32_t seen = 0;                      // bits 0..3: chunks of 16 inputs, 4: a weight that is no power of two, 8..: weights
-      if (r < o)
-        for (int k = t & 7; k < in; k += 8) {
-          const float w = W[off + r * in + k], x = fabsf(w) * mb[k];
-          sum += x;  // (a weight that is not finite shows here, whatever its input)
-          if (w == 0.f || mb[k] == 0.f) continue;
-          sq = fmaf(x, x, sq);
-          pos += w > 0.f ? x : 0.f;
-          top = fmaxf(top, ldexpf(fabsf(w), -S.a[l][k]));
-          seen = (seen | 1u << (k >> 4) | ((__float_as_uint(w) & 0x7FFFFFu) || l == 0 ? 16u : 0u)) + 256u;
-        }
+      uint32_t seen = 0;                     // bits 0..3: chunks of 16 inputs, 4: a weight that is no power of two, 8..: weights
+      float w[kHid / 8];
+      const float b = r < o && l < nhid ? B[boff + r] : 0.f;
+#pragma unroll
+      for (int j = 0; j < kHid / 8; ++j) {
+        const int k = (t & 7) + 8 * j;
+        w[j] = r < o && k < in ? W[off + r * in + k] : 0.f;
+      }
+#pragma unroll
+      for (int j = 0; j < kHid / 8; ++j) {
+        const int k = (t & 7) + 8 * j;
+        if (w[j] == 0.f) continue;
+        const float x = fabsf(w[j]) * mb[k];
+        sum += x;  // (a weight that is not finite shows here, whatever its input)
+        if (mb[k] == 0.f) continue;
+        sq = fmaf(x, x, sq);
+        pos += w[j] > 0.f ? x : 0.f;
+        top = fmaxf(top, fabsf(w[j]) * S.down[l][k]);
+        seen = (seen | 1u << (k >> 4) | ((__float_as_uint(w[j]) & 0x7FFFFFu) || l == 0 ? 16u : 0u)) + 256u;
+      }
 #pragma unroll
       for (int d = 1; d < 8; d <<= 1) {
         sum += __shfl_xor_sync(0xffffffffu, sum, d);
@@ -116,11 +130,10 @@ __device__ inline void f32s_scales(const float* __restrict__ W, const float* __r
         seen = ((seen | other) & 31u) | ((seen & ~31u) + (other & ~31u));
       }
       if (r < o && (t & 7) == 0) {
-        const float b = l < nhid ? B[boff + r] : 0.f;
         // share of the inputs that carry the row, and how far they have one sign
         const float many = sq > 0.f ? sum * rsqrtf(sq) : 0.f;
-        const float one_sign = sum > 0.f ? fabsf(2.f * pos - sum) / sum : 0.f;
-        const float coherent = many * many / (float)in * one_sign;
+        const float one_sign = sum > 0.f ? __fdividef(fabsf(2.f * pos - sum), sum) : 0.f;
+        const float coherent = many * many * (l == 0 ? 1.f / 12.f : inv_hid) * one_sign;
         sum += fabsf(b);
         if (!(sum < 1e30f) || !(top < 1e30f)) S.bad = 1;  // (also NaN)
         // the margin covers the FP32 rounding of these sums
@@ -132,8 +145,10 @@ __device__ inline void f32s_scales(const float* __restrict__ W, const float* __r
           if (b != 0.f) a = min(a, 15 - exponent_above(fabsf(b)));
           a = min(max(a, -120), 120);
         }
+        const bool dead = l < nhid && !(bound > 0.f);
         S.bound[(l + 1) & 1][r] = 1.0001f * bound;
-        S.a[l + 1][r] = l < nhid && !(bound > 0.f) ? kF32sDead : (short)a;
+        S.up[l + 1][r] = dead ? 0.f : pow2f(a);
+        S.down[l + 1][r] = dead ? 0.f : pow2f(-a);
         const int n = l == 0 ? 1 : __popc(seen & 15u);
         const bool lone = (seen >> 8) <= 1 && !(seen & 16u) && b == 0.f;
         S.loss[l + 1][r] = lone ? 0.f : 0.5f * (float)(n + 1) * (kTruncUlp + kAlignUlp * coherent) * 1.1920929e-7f;
@@ -145,59 +160,71 @@ __device__ inline void f32s_scales(const float* __restrict__ W, const float* __r
   }
 }
 
-// The image (see TcLayout; already cleared) from the FP32 MLP and the scales.
-__device__ inline void f32s_pack(unsigned char* img, const TcLayout L, const float* __restrict__ W,
-                                 const float* __restrict__ B, int hid, int nout, int t, int nt, const F32sScratch& S) {
+// The image (see TcLayout; already cleared) from the FP32 MLP and the scales, two
+// weights of a row at a time.
+static __device__ __noinline__ void f32s_pack(unsigned char* img, const TcLayout L, const float* __restrict__ W,
+                                              const float* __restrict__ B, int hid, int nout, int t, int nt,
+                                              const F32sScratch& S) {
   const int nhid = L.nhid, R1 = L.w1_row();
-  auto split = [](double w, uint16_t (&part)[3]) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const __half h = __float2half_rn((float)w);
-      part[i] = __half_as_ushort(h);
-      w -= (double)__half2float(h);
-    }
+  // parts of w + w c, exact to 2^-36 of it
+  auto split = [](float w, float c, uint32_t (&part)[3]) {
+    const __half h = __float2half_rn(fmaf(w, c, w));
+    const float r = fmaf(w, c, w - __half2float(h));  // (the difference is exact)
+    const __half lo = __float2half_rn(r);
+    part[0] = __half_as_ushort(h);
+    part[1] = __half_as_ushort(lo);
+    part[2] = __half_as_ushort(__float2half_rn(r - __half2float(lo)));
   };
-  auto put = [&](uint32_t at, uint16_t v) { *reinterpret_cast<uint16_t*>(img + at) = v; };
-  auto raise = [&](int l, int i) { return 1.0 + (double)S.loss[l][i]; };
+  auto put = [&](uint32_t at, uint32_t v) { *reinterpret_cast<uint16_t*>(img + at) = (uint16_t)v; };
+  auto put2 = [&](uint32_t at, uint32_t v0, uint32_t v1) { *reinterpret_cast<uint32_t*>(img + at) = v0 | v1 << 16; };
+  const int sh = hid == 16 ? 3 : hid == 32 ? 4 : 5;  // log2 of a hidden row's pairs
   int off = 0, boff = 0;
   for (int l = 0; l <= nhid; ++l) {
-    const int in = l == 0 ? 12 : hid, o = l == nhid ? nout : hid;
-    for (int i = t; i < in * o; i += nt) {
-      const int n = i / in, k = i - n * in;
-      if (S.a[l + 1][n] == kF32sDead || S.a[l][k] == kF32sDead) continue;  // (the image is cleared)
-      uint16_t q[3];
-      const float w = ldexpf(W[off + i], S.a[l + 1][n] - S.a[l][k]);
-      split((l == 0 ? 256.0 / 255.0 : 1.0) * raise(l + 1, n) * w, q);
-      if (l == 0) {
+    const int o = l == nhid ? nout : hid;
+    if (l == 0) {
+      for (int i = t; i < 6 * o; i += nt) {
+        const int n = i / 6, k = 2 * (i - 6 * n);
+        const float up = S.up[1][n] * S.down[0][0], e = S.loss[1][n], c = 1.f / 255.f + e * (256.f / 255.f);
+        uint32_t q[3], q1[3];
+        split(W[12 * n + k] * up, c, q);
+        split(W[12 * n + k + 1] * up, c, q1);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) put(L.off_w1() + off_ilv(n, 2 * (16 * j + k), R1), q[j]);
-      } else {
-        const int base = l == nhid ? L.off_wo() : L.off_wh(l - 1);
-        const int part = l == nhid ? L.wo_part() : L.wh_part();
-        put(base + off_sw128(n, 2 * k), q[0]);
-        put(base + off_sw128(n, 2 * k) + part, q[1]);
+        for (int j = 0; j < 3; ++j) put2(L.off_w1() + off_ilv(n, 2 * (16 * j + k), R1), q[j], q1[j]);
       }
+      off += 12 * o;
+    } else {
+      const int base = l == nhid ? L.off_wo() : L.off_wh(l - 1), part = l == nhid ? L.wo_part() : L.wh_part();
+#pragma unroll 4
+      for (int i = t; i < o << sh; i += nt) {
+        const int n = i >> sh, k = 2 * (i & ((1 << sh) - 1));
+        const float* w = W + off + n * hid + k;
+        const float up = S.up[l + 1][n], e = S.loss[l + 1][n];
+        uint32_t q[3], q1[3];
+        split(w[0] * S.down[l][k] * up, e, q);
+        split(w[1] * S.down[l][k + 1] * up, e, q1);
+        const uint32_t at = base + off_sw128(n, 2 * k);
+        put2(at, q[0], q1[0]);
+        put2(at + part, q[1], q1[1]);
+      }
+      off += hid * o;
     }
     for (int i = t; i < o && l < nhid; i += nt) {
-      if (S.a[l + 1][i] == kF32sDead) continue;
-      uint16_t q[3];
-      split(raise(l + 1, i) * ldexpf(B[boff + i], S.a[l + 1][i]), q);
+      uint32_t q[3];
+      split(B[boff + i] * S.up[l + 1][i], S.loss[l + 1][i], q);
       if (l == 0) {
 #pragma unroll
         for (int j = 0; j < 3; ++j) put(L.off_w1() + off_ilv(i, 2 * (16 * j + 12), R1), q[j]);
       } else {
-        put(L.off_bth(l - 1) + off_interleave(i, 0), q[0]);
-        put(L.off_bth(l - 1) + off_interleave(i, 2), q[1]);
+        put2(L.off_bth(l - 1) + off_interleave(i, 0), q[0], q[1]);
       }
     }
-    off += in * o;
     boff += o;
   }
   // output biases, then (at nhid kHid) the multipliers of the accumulated products
   float* out = reinterpret_cast<float*>(img + L.off_bias());
   for (int c = t; c < kOutPad; c += nt) {
     out[c] = c < nout ? B[nhid * hid + c] : 0.f;
-    out[nhid * kHid + c] = c < nout ? ldexpf(1.f, -S.a[nhid + 1][c]) : 0.f;
+    out[nhid * kHid + c] = c < nout ? S.down[nhid + 1][c] : 0.f;
   }
 }
 
