@@ -16,8 +16,9 @@ constexpr int kMaxOut = 16;
 // Operand forms of the tensor-core decode.  The split forms carry every weight
 // and activation as a pair hi + lo of the narrow format and run three products
 // per layer into one FP32 accumulator: hi(A) hi(W) + lo(A) hi(W) + hi(A) lo(W).
-// kF32Split is kF16Split with the output layer's FP32 accumulator written as
-// FP32 (no output rounding): the FP32-accurate form.
+// kF32Split, the FP32-accurate form, is kF16Split with scaled neurons, lo(A) lo(W), a
+// third part of layer 1's operands and the output layer's FP32 accumulator written
+// as FP32 (f32s_pack.cuh).
 enum TcForm { kF16 = 0, kF8 = 1, kF16Split = 2, kF8Split = 3, kF32Split = 4 };
 
 // Bytes of per-warp output staging: 32 texels x up to 16 channels of FP16, or FP32,
